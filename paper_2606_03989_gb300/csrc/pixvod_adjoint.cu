@@ -210,11 +210,11 @@ __global__ void __launch_bounds__(TILE_PX) k_adjoint_fwd(const AdjArgs A, T* __r
     for (int q = 0; q < 6; ++q) e[q] = w[q] = T(0);
     if (inside && c.has[k]) {
         set_scales(A, io);
-        T xi[6], R[9], t[3];
+        T xi[6], qi[4], t[3];
         for (int q = 0; q < 6; ++q) xi[q] = io.mu(q);
-        se3_exp(xi, R, t);
+        se3_exp_q(xi, qi, t);
         hw::IdFwd<T> f;
-        hw::damped_identity(io, c, k, R, t, L, e, &f);
+        hw::damped_identity_at(io, c, k, qi, t, L, e, &f);
         hw::identity_w(io, k, L, w);
         for (int q = 0; q < 21; ++q) sp[(SCR_FWD + 27 * k + q) * TILE_PX] = L[q];
         for (int q = 0; q < 6; ++q) sp[(SCR_FWD + 27 * k + 21 + q) * TILE_PX] = e[q];

@@ -314,71 +314,6 @@ struct PixCtx {
     bool clamp_x, clamp_y;  // the warped coordinate was clamped into the image
 };
 
-// The identity message of direction k (Eq. 5 through the 12-D Schur complement,
-// in the sweep kernel's product form), undamped: Lambda_new (packed) and eta_new.
-// Also returns what the reverse pass needs: rb, W, the factor L of
-// A = W + lam_R I (with 1/L_ii on its diagonal), z = A^-1 u, iuz = 1/(1 + u^T z).
-template <typename T>
-PV_HD void identity_message(const T* nb, const T* R, const T* t, T lam_R, T* rb, T* W, T* L, T* z, T* iuz_out,
-                            T* Lnew, T* enew) {
-    {
-        T Rj[9], tj[3], Rr[9], tr[3];
-        se3_exp(nb + NB_XJ, Rj, tj);
-        se3_invmul(Rj, tj, R, t, Rr, tr);
-        se3_log(Rr, tr, rb);
-    }
-    T gv[6], uj[6];
-    for (int q = 0; q < 21; ++q) {
-        W[q] = nb[NB_MP + q] - nb[NB_ML + q];
-        L[q] = W[q];
-    }
-    for (int q = 0; q < 6; ++q) {
-        uj[q] = nb[NB_U + q];
-        T wr = T(0);
-        for (int c = 0; c < 6; ++c) wr += W[pidx(q, c)] * rb[c];
-        gv[q] = -nb[NB_ME + q] - wr;
-    }
-    for (int q = 0; q < 6; ++q) L[pidx(q, q)] += lam_R;
-    T idg[6];
-    chol_packed<6>(L, idg);
-    for (int q = 0; q < 6; ++q) z[q] = uj[q];
-    fwd_solve<6>(L, idg, z);
-    bwd_solve<6>(L, idg, z);
-    fwd_solve<6>(L, idg, gv);
-    bwd_solve<6>(L, idg, gv);
-    T uz = T(0), ur = T(0), uh = T(0);
-    for (int q = 0; q < 6; ++q) {
-        uz += uj[q] * z[q];
-        ur += uj[q] * rb[q];
-        uh += uj[q] * gv[q];
-        L[pidx(q, q)] = idg[q];
-    }
-    const T iuz = v_div(T(1), T(1) + uz);
-    const T crank = lam_R * lam_R * iuz;
-    const T ecoef = (ur + uh) * iuz;
-    for (int q = 0; q < 6; ++q) enew[q] = lam_R * (gv[q] - ecoef * z[q]);
-    for (int c = 0; c < 6; ++c) {
-        T x[6];
-        for (int r = 0; r < 6; ++r) x[r] = W[pidx(r, c)];
-        fwd_solve_id<6>(L, x);
-        bwd_solve_id<6>(L, x);
-        for (int r = c; r < 6; ++r) Lnew[pidx(r, c)] = lam_R * x[r] + crank * z[r] * z[c];
-    }
-    *iuz_out = iuz;
-}
-
-// C^-1 x with C = A + u u^T, A = L L^T (1/L_ii on the diagonal), z = A^-1 u
-template <typename T>
-PV_HD void solve_C(const T* L, const T* z, T iuz, const T* u, const T* x, T* y) {
-    for (int q = 0; q < 6; ++q) y[q] = x[q];
-    fwd_solve_id<6>(L, y);
-    bwd_solve_id<6>(L, y);
-    T uy = T(0);
-    for (int q = 0; q < 6; ++q) uy += u[q] * y[q];
-    const T s = uy * iuz;
-    for (int q = 0; q < 6; ++q) y[q] -= s * z[q];
-}
-
 // Photometric factor (Eqs. 2, 3) at the current mean with the recorded validity
 // and Huber branch: J (7), alpha, r. Also the intermediate values the reverse
 // pass needs.
@@ -445,40 +380,52 @@ struct IdFwd {
 };
 constexpr int ID_FWD_VALS = 54;
 
-// C^-1 (packed) from the factor of A = W + lam_R I, z = A^-1 u, 1/(1 + u^T z):
-// six solves on the unit vectors
-template <typename T>
-PV_HD void form_Ci(const T* L, const T* z, T iuz, const T* u, T* Ci) {
-#pragma unroll
-    for (int cc = 0; cc < 6; ++cc) {
-        T ec[6], o[6];
-        for (int r = 0; r < 6; ++r) ec[r] = r == cc ? T(1) : T(0);
-        solve_C(L, z, iuz, u, ec, o);
-        for (int r = cc; r < 6; ++r) Ci[pidx(r, cc)] = o[r];
-    }
-}
-
-// The damped identity message of direction k into the pixel at pose (R, t):
-// Lambda (packed) and eta, from the neighbour's values and the pixel's old
-// message of slot k; with f, also what its reverse pass needs.
+// The damped identity message of direction k into the pixel at pose (q, t) =
+// Exp(io.mu): Lambda (packed) and eta, from the neighbour's values and the pixel's
+// old message of slot k, with the sweep kernel's operations; with f, also what its
+// reverse pass needs.
 template <typename T, typename IO>
-PV_HD void damped_identity(IO& io, const PixCtx<T>& c, int k, const T* R, const T* t, T* L, T* e,
-                           IdFwd<T>* f = nullptr) {
+PV_HD void damped_identity_at(IO& io, const PixCtx<T>& c, int k, const T* qi, const T* t, T* L, T* e,
+                              IdFwd<T>* f = nullptr) {
     const T beta = c.beta, omb = T(1) - c.beta;
-    T nbk[NB_VALS];
-    for (int q = 0; q < NB_VALS; ++q) nbk[q] = io.nb(k, q);
-    T rb[6], W[21], Lc[21], z[6], iuz, Ln[21], en[6];
-    identity_message(nbk, R, t, c.lam_R, rb, W, Lc, z, &iuz, Ln, en);
-    for (int q = 0; q < 6; ++q) e[q] = omb * en[q] + beta * io.msg(k, 21 + q);
-    for (int q = 0; q < 21; ++q) L[q] = omb * Ln[q] + beta * io.msg(k, q);
+    T xj[6], W[21], uj[6], ev[6], rb[6];
+    for (int q = 0; q < 6; ++q) xj[q] = io.nb(k, NB_XJ + q);
+    for (int q = 0; q < 21; ++q) W[q] = io.nb(k, NB_MP + q) - io.nb(k, NB_ML + q);
+    for (int q = 0; q < 6; ++q) {
+        uj[q] = io.nb(k, NB_U + q);
+        ev[q] = -io.nb(k, NB_ME + q);
+    }
+    se3_between(xj, qi, t, rb);
+    IdMsg<T> m;
+    identity_msg(W, uj, ev, rb, c.lam_R, m);
+    const T wl = omb * c.lam_R, wll = wl * c.lam_R;
+    for (int q = 0; q < 6; ++q) e[q] = v_fma(wl, m.he[q], beta * io.msg(k, 21 + q));
+#pragma unroll
+    for (int r = 0; r < 6; ++r)
+#pragma unroll
+        for (int cc = 0; cc <= r; ++cc) L[pidx(r, cc)] = m.lambda(r, cc, wl, wll, beta * io.msg(k, pidx(r, cc)));
     if (f) {
         for (int q = 0; q < 6; ++q) {
             f->rb[q] = rb[q];
-            f->en[q] = en[q];
+            f->en[q] = c.lam_R * m.he[q];
         }
         for (int q = 0; q < 21; ++q) f->W[q] = W[q];
-        form_Ci(Lc, z, iuz, nbk + NB_U, f->Ci);
+#pragma unroll
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+            for (int cc = 0; cc <= r; ++cc) f->Ci[pidx(r, cc)] = m.ci(r, cc);
     }
+}
+
+// The same for a caller that holds the pose as (R, t) = Exp(io.mu): the message is
+// formed from io.mu's quaternion.
+template <typename T, typename IO>
+PV_HD void damped_identity(IO& io, const PixCtx<T>& c, int k, const T* /*R*/, const T* /*t*/, T* L, T* e,
+                           IdFwd<T>* f = nullptr) {
+    T xi[6], qi[4], t[3];
+    for (int q = 0; q < 6; ++q) xi[q] = io.mu(q);
+    se3_exp_q(xi, qi, t);
+    damped_identity_at(io, c, k, qi, t, L, e, f);
 }
 
 // The adjoint of the projected eta_k' = eta_k - Lambda_k tau reaches tau as

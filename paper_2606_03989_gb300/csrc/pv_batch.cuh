@@ -101,7 +101,7 @@ __device__ __forceinline__ bool grid_sync(const GridSync& gs) {
 //    publishes the stores.
 // work == nullptr stands for the tiles of sequence 0 in order.
 template <typename T>
-__global__ void __launch_bounds__(SWEEP_THREADS, 4) k_sweeps(const SeqDesc<T>* __restrict__ seqs,
+__global__ void __launch_bounds__(SWEEP_THREADS, sizeof(T) == 4 ? 4 : 2) k_sweeps(const SeqDesc<T>* __restrict__ seqs,
                                                              const Work* __restrict__ work, int n_work,
                                                              int n_iters, int cur0, GridSync gs) {
     // msg[p * TILE_PX + tid]: a tile's 108 identity-message planes, bulk-copied in

@@ -313,8 +313,8 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
 #pragma unroll
     for (int k = 0; k < 6; ++k) xi[k] = ld_state(Si + k * TILE_PX);
     d = ld_state(Si + 6 * TILE_PX);
-    T R[9], t[3];
-    se3_exp(xi, R, t);
+    T qi[4], t[3];
+    se3_exp_q(xi, qi, t);
 
     // The belief has the exact structure
     //   Lambda_b = blockdiag(M_p, m_d) + alpha J J^T,  eta_b = eta_o - alpha r J
@@ -362,9 +362,7 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
         // eta_v = -eta_{f->j}. All of j's loads are issued here, ahead of the Exp/Log
         // chain of the residual, so that their latency overlaps it.
         const T* mj = Sj + (PL_ID + ID_STRIDE * ko) * TILE_PX;
-        T W[21], C[21], z[6], gv[6];
-        T uz = T(0), ur = T(0), uh = T(0);
-        T uj[6], xj[6];
+        T W[21], uj[6], gv[6], xj[6];
 #pragma unroll
         for (int q = 0; q < 6; ++q) xj[q] = ld_state(Sj + q * TILE_PX);
 #pragma unroll
@@ -374,74 +372,26 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
             uj[q] = ld_state(Sj + (PL_U + q) * TILE_PX);
             gv[q] = -ld_state(mj + (21 + q) * TILE_PX);
         }
-        // identity factor (Eq. 5): r = Log(Exp(xi_j)^-1 Exp(xi_i)), J_i = I, J_j = -I
         T rb[6];
-        {
-            T Rj[9], tj[3], Rr[9], tr[3];
-            se3_exp(xj, Rj, tj);
-            se3_invmul(Rj, tj, R, t, Rr, tr);
-            se3_log(Rr, tr, rb);
-        }
-        {
-#pragma unroll
-            for (int q = 0; q < 21; ++q) C[q] = W[q];
-            // g0 = eta_v - W r
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                T wr = T(0);
-#pragma unroll
-                for (int c = 0; c < 6; ++c) wr += W[pidx(q, c)] * rb[c];
-                gv[q] -= wr;
-            }
-            // A = W + lam_R I is well conditioned (its eigenvalues are at least lam_R);
-            // the rank-one u u^T, which can be far larger, stays out of the factorisation
-#pragma unroll
-            for (int q = 0; q < 6; ++q) C[pidx(q, q)] += F.lam_R;
-            T idg0[6];
-            if (!chol_packed<6>(C, idg0)) flags |= FLAG_NONPOS_PIVOT;
-#pragma unroll
-            for (int q = 0; q < 6; ++q) z[q] = uj[q];
-            fwd_solve<6>(C, idg0, z);
-            bwd_solve<6>(C, idg0, z);   // z = A^-1 u
-            fwd_solve<6>(C, idg0, gv);
-            bwd_solve<6>(C, idg0, gv);  // h = A^-1 g0
-#pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                uz += uj[q] * z[q];
-                ur += uj[q] * rb[q];
-                uh += uj[q] * gv[q];
-                C[pidx(q, q)] = idg0[q];  // keep 1/L_qq on the diagonal (the solves below read it there)
-            }
-        }
-        const T iuz = v_div(T(1), T(1) + uz);
-        const T crank = F.lam_R * F.lam_R * iuz;
-        // with C = A + u u^T (Sherman-Morrison):
-        // eta_msg = lam_R C^-1 (eta_v - V r) = lam_R (h - z (u^T r + u^T h) / (1 + u^T z))
-        const T ecoef = (ur + uh) * iuz;
+        se3_between(xj, qi, t, rb);
+        IdMsg<T> m;
+        if (!identity_msg(W, uj, gv, rb, F.lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
+        // damped: (1 - beta) new + beta old, over the old message in shared memory
+        const T wl = omb * F.lam_R, wll = wl * F.lam_R;
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
-            T e = omb * (F.lam_R * (gv[q] - ecoef * z[q])) + beta * mb[(21 + q) * TILE_PX];
+            const T e = v_fma(wl, m.he[q], beta * mb[(21 + q) * TILE_PX]);
             eb[q] += e;
             mb[(21 + q) * TILE_PX] = e;
         }
-        // Lambda_msg = lam_R C^-1 V = lam_R A^-1 W + lam_R^2 / (1 + u^T z) z z^T, the first
-        // term (equal to W - W A^-1 W) one column at a time, rows c..5 of column c; this
-        // product form has no cancellation for W << lam_R (~ W) or W >> lam_R (~ lam_R I)
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            T x[6];
-#pragma unroll
-            for (int r = 0; r < 6; ++r) x[r] = W[pidx(r, c)];
-            fwd_solve_id<6>(C, x);
-            bwd_solve_id<6>(C, x);
+        for (int c = 0; c < 6; ++c)
 #pragma unroll
             for (int r = c; r < 6; ++r) {
-                T l = omb * (F.lam_R * x[r] + crank * z[r] * z[c]) + beta * mb[pidx(r, c) * TILE_PX];
+                const T l = m.lambda(r, c, wl, wll, beta * mb[pidx(r, c) * TILE_PX]);
                 Mp[pidx(r, c)] += l;
                 mb[pidx(r, c) * TILE_PX] = l;
             }
-        }
-
     }
 
     // normal-integration factors (Eq. 6): r_i = d_i - d_j + sg m
@@ -478,6 +428,8 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
     // --- a1: photometric factor (Eqs. 2, 3) at the current mean (it enters only
     // the belief below, so it is evaluated after the pairwise messages) ---
     {
+        T R[9];
+        quat_matrix(qi, R);
         T z = v_exp(d);
         T Xs[3] = {z * (T(u) - g.cx) * g.ifx, z * (T(v) - g.cy) * g.ify, z};
         T Xt[3];
@@ -589,10 +541,8 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
     if (a.br) a.br[tile * TILE_PX + tid] = br;
     // mu <- mu (+) tau
     {
-        T Rt[9], tt[3], Rn[9], tn[3], xn[6];
-        se3_exp(tau, Rt, tt);
-        se3_mul(R, t, Rt, tt, Rn, tn);
-        se3_log(Rn, tn, xn);
+        T xn[6];
+        se3_update(qi, t, tau, xn);
 #pragma unroll
         for (int q = 0; q < 6; ++q) Di[q * TILE_PX] = xn[q];
         Di[6 * TILE_PX] = d + tau[6];

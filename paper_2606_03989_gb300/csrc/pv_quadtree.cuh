@@ -50,67 +50,6 @@ __host__ __device__ inline int qt_node(const QtGeom& q, int level, int r, int c)
     return q.base[level - 1] + r * q.w[level - 1] + c;
 }
 
-// Message to a receiver from an identity factor (Eq. 5, J = +I for the receiver,
-// -I for the sender), given the sender's variable-to-factor marginal
-// V = W + u u^T, eta_v (u = 0 for a pose node) and the residual
-// rb = Log(Exp(xi_sender)^-1 Exp(xi_receiver)) at the current means:
-//   Lambda = lam C^-1 V = lam A^-1 W + lam^2 / (1 + u^T z) z z^T,
-//   eta = lam C^-1 (eta_v - V rb),  A = W + lam I, C = A + u u^T, z = A^-1 u.
-// (The grid sweep uses the same algebra, inline.)
-template <typename T>
-__device__ void identity_message(const T* W, const T* u, const T* etav, const T* rb, T lam, T* Lout, T* eout,
-                                 unsigned* flags) {
-    T C[21], z[6], gv[6], idg[6];
-#pragma unroll
-    for (int q = 0; q < 21; ++q) C[q] = W[q];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        T wr = T(0);
-#pragma unroll
-        for (int c = 0; c < 6; ++c) wr += W[pidx(q, c)] * rb[c];
-        gv[q] = etav[q] - wr;
-        C[pidx(q, q)] += lam;
-        z[q] = u[q];
-    }
-    if (!chol_packed<6>(C, idg)) *flags |= FLAG_NONPOS_PIVOT;
-    fwd_solve<6>(C, idg, z);
-    bwd_solve<6>(C, idg, z);
-    fwd_solve<6>(C, idg, gv);
-    bwd_solve<6>(C, idg, gv);
-    T uz = T(0), ur = T(0), uh = T(0);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-        uz += u[q] * z[q];
-        ur += u[q] * rb[q];
-        uh += u[q] * gv[q];
-        C[pidx(q, q)] = idg[q];
-    }
-    const T iuz = v_div(T(1), T(1) + uz);
-    const T crank = lam * lam * iuz;
-    const T ecoef = (ur + uh) * iuz;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) eout[q] = lam * (gv[q] - ecoef * z[q]);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        T x[6];
-#pragma unroll
-        for (int r = 0; r < 6; ++r) x[r] = W[pidx(r, c)];
-        fwd_solve_id<6>(C, x);
-        bwd_solve_id<6>(C, x);
-#pragma unroll
-        for (int r = c; r < 6; ++r) Lout[pidx(r, c)] = lam * x[r] + crank * z[r] * z[c];
-    }
-}
-
-// rb = Log(Exp(xi_s)^-1 Exp(xi_r)) from the receiver's (R, t) and the sender's mean
-template <typename T>
-__device__ __forceinline__ void identity_residual(const T* R, const T* t, const T* xi_s, T* rb) {
-    T Rs[9], ts[3], Rr[9], tr[3];
-    se3_exp(xi_s, Rs, ts);
-    se3_invmul(Rs, ts, R, t, Rr, tr);
-    se3_log(Rr, tr, rb);
-}
-
 // One pixel's sweep update: as the grid sweep (priors, normal-integration messages
 // from the four grid neighbours, photometric factor, structured belief solve,
 // mu (+) tau, projected stores), with the identity message coming only from the
@@ -130,8 +69,8 @@ __device__ __forceinline__ void qt_pixels(const QtArgs<T>& a, int bx, int by) {
 #pragma unroll
     for (int k = 0; k < 6; ++k) xi[k] = Si[k * TILE_PX];
     const T d = Si[6 * TILE_PX];
-    T R[9], t[3];
-    se3_exp(xi, R, t);
+    T qi[4], t[3];
+    se3_exp_q(xi, qi, t);
     T eb[7], Mp[21];
 #pragma unroll
     for (int q = 0; q < 7; ++q) eb[q] = T(0);
@@ -164,17 +103,22 @@ __device__ __forceinline__ void qt_pixels(const QtArgs<T>& a, int bx, int by) {
         for (int c = 0; c < 21; ++c) W[c] = N[(NP_M + c) * st] - mk[c * st];
 #pragma unroll
         for (int c = 0; c < 6; ++c) ev[c] = -mk[(21 + c) * st];
-        identity_residual(R, t, xs, rb);
-        identity_message(W, zero6, ev, rb, F.lam_R, Lnew, enew6, &flags);
+        se3_between(xs, qi, t, rb);
+        IdMsg<T> m;
+        if (!identity_msg(W, zero6, ev, rb, F.lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
         const T* old = Si + PL_ID * TILE_PX;
+        const T wl = omb * F.lam_R, wll = wl * F.lam_R;
 #pragma unroll
-        for (int c = 0; c < 21; ++c) {
-            Lnew[c] = omb * Lnew[c] + beta * old[c * TILE_PX];
-            Mp[c] += Lnew[c];
-        }
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+            for (int c = 0; c <= r; ++c) {
+                const T l = m.lambda(r, c, wl, wll, beta * old[pidx(r, c) * TILE_PX]);
+                Lnew[pidx(r, c)] = l;
+                Mp[pidx(r, c)] += l;
+            }
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
-            enew6[c] = omb * enew6[c] + beta * old[(21 + c) * TILE_PX];
+            enew6[c] = v_fma(wl, m.he[c], beta * old[(21 + c) * TILE_PX]);
             eb[c] += enew6[c];
         }
     }
@@ -206,6 +150,8 @@ __device__ __forceinline__ void qt_pixels(const QtArgs<T>& a, int bx, int by) {
 #pragma unroll
     for (int q = 0; q < 7; ++q) J[q] = T(0);
     {
+        T R[9];
+        quat_matrix(qi, R);
         const T z = v_exp(d);
         const T Xs[3] = {z * (T(u) - g.cx) * g.ifx, z * (T(v) - g.cy) * g.ify, z};
         T Xt[3];
@@ -296,10 +242,8 @@ __device__ __forceinline__ void qt_pixels(const QtArgs<T>& a, int bx, int by) {
         for (int q = 0; q < 7; ++q) tau[q] = T(0);
     }
     {
-        T Rt[9], tt[3], Rn[9], tn[3], xn[6];
-        se3_exp(tau, Rt, tt);
-        se3_mul(R, t, Rt, tt, Rn, tn);
-        se3_log(Rn, tn, xn);
+        T xn[6];
+        se3_update(qi, t, tau, xn);
 #pragma unroll
         for (int q = 0; q < 6; ++q) Di[q * TILE_PX] = xn[q];
         Di[6 * TILE_PX] = d + tau[6];
@@ -482,17 +426,20 @@ __device__ __forceinline__ void qt_node_msgs(const QtArgs<T>& a, int blk) {
         for (int m = 0; m < ID_STRIDE; ++m) dst[m * st] = T(0);
         return;
     }
-    T R[9], t[3];
-    se3_exp(xi, R, t);
+    T qi[4], t[3], rb[6];
+    se3_exp_q(xi, qi, t);
+    se3_between(xs, qi, t, rb);
     unsigned flags = 0;
-    T rb[6], L[21], e[6];
-    identity_residual(R, t, xs, rb);
-    identity_message(W, u, ev, rb, lam, L, e, &flags);
-    const T beta = F.beta, omb = T(1) - F.beta;
+    IdMsg<T> im;
+    if (!identity_msg(W, u, ev, rb, lam, im)) flags |= FLAG_NONPOS_PIVOT;
+    const T beta = F.beta, wl = (T(1) - F.beta) * lam, wll = wl * lam;
 #pragma unroll
-    for (int m = 0; m < 21; ++m) dst[m * st] = omb * L[m] + beta * ov[m];
+    for (int rr = 0; rr < 6; ++rr)
 #pragma unroll
-    for (int m = 0; m < 6; ++m) dst[(21 + m) * st] = omb * e[m] + beta * ov[21 + m];
+        for (int cc = 0; cc <= rr; ++cc)
+            dst[pidx(rr, cc) * st] = im.lambda(rr, cc, wl, wll, beta * ov[pidx(rr, cc)]);
+#pragma unroll
+    for (int m = 0; m < 6; ++m) dst[(21 + m) * st] = v_fma(wl, im.he[m], beta * ov[21 + m]);
     if (flags) atomicOr(&a.sc->flags, flags);
 }
 
@@ -509,10 +456,10 @@ __device__ __forceinline__ void qt_node_belief(const QtArgs<T>& a, int blk) {
     const NodePos p = node_pos(q, n);
     const T* N = a.nin + n;
     T* O = a.nout + n;
-    T xi[6], R[9], t[3];
+    T xi[6], qi[4], t[3];
 #pragma unroll
     for (int k = 0; k < 6; ++k) xi[k] = N[(NP_MU + k) * st];
-    se3_exp(xi, R, t);
+    se3_exp_q(xi, qi, t);
     const T lamP = F.lam_P * level_scale<T>(p.lvl) * T(4);     // sigma_P / 2^l
     T Mb[21], eb[6];
 #pragma unroll
@@ -549,10 +496,8 @@ __device__ __forceinline__ void qt_node_belief(const QtArgs<T>& a, int blk) {
         for (int k = 0; k < 6; ++k) tau[k] = T(0);
     }
     {
-        T Rt[9], tt[3], Rn[9], tn[3], xn[6];
-        se3_exp(tau, Rt, tt);
-        se3_mul(R, t, Rt, tt, Rn, tn);
-        se3_log(Rn, tn, xn);
+        T xn[6];
+        se3_update(qi, t, tau, xn);
 #pragma unroll
         for (int k = 0; k < 6; ++k) O[(NP_MU + k) * st] = xn[k];
     }
