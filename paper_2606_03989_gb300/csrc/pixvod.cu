@@ -309,6 +309,31 @@ cudaError_t sweep_attributes() {
     return once;
 }
 
+// launch on `st` with programmatic stream serialization: the kernel may be
+// scheduled while its predecessor drains (it waits for it itself, pv::pdl_wait)
+template <typename... P, typename... A>
+void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // the error is read by cudaGetLastError
+}
+
+// one synchronous grid sweep: the tiles of `work` (null: of the descriptor's
+// sequence in order; from the end when `flip` is odd), reading state buffer `cur`
+template <typename T>
+void launch_sweep(const pv::SeqDesc<T>* desc, const pv::Work* work, int n_work, int cur, int flip, cudaStream_t st) {
+    launch_pdl(pv::k_sweeps<T>, dim3(n_work), sweep_block(), pv::sweep_smem_bytes<T>(), st, desc, work, n_work, 1, cur,
+               flip, pv::GridSync{nullptr, nullptr, nullptr, 0});
+}
+
 pixvod_status cuda_status(cudaError_t e) {
     if (e == cudaSuccess) return PIXVOD_OK;
     fprintf(stderr, "pixvod: CUDA error %s\n", cudaGetErrorString(e));
@@ -457,8 +482,7 @@ pixvod_status run_sweeps(pixvod_handle* h, int n) {
         if (is_quadtree(h)) {
             s = launch_qt_sweep<T>(h);
         } else {
-            pv::k_sweeps<T><<<n_tiles, sweep_block(), pv::sweep_smem_bytes<T>(), h->stream>>>(
-                desc_ptr<T>(h), nullptr, n_tiles, 1, h->cur, pv::GridSync{nullptr, nullptr, nullptr, 0});
+            launch_sweep<T>(desc_ptr<T>(h), nullptr, n_tiles, h->cur, h->cur, h->stream);
             s = launched(h);
         }
         if (prof) {
@@ -509,8 +533,7 @@ pixvod_status run_sweeps_recorded(pixvod_handle* h, int n) {
         if (s != PIXVOD_OK) return s;
         const pv::SeqDesc<T>* dd = reinterpret_cast<const pv::SeqDesc<T>*>(h->rec_ws + R.off_desc);
         for (int c = 1; c <= n; ++c) {
-            pv::k_sweeps<T><<<n_tiles, sweep_block(), pv::sweep_smem_bytes<T>(), h->stream>>>(
-                dd + (c - 1), nullptr, n_tiles, 1, 0, pv::GridSync{nullptr, nullptr, nullptr, 0});
+            launch_sweep<T>(dd + (c - 1), nullptr, n_tiles, 0, c, h->stream);
             if ((s = launched(h)) != PIXVOD_OK) return s;
         }
         h->cur = cur0 ^ 1;
@@ -712,8 +735,7 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
         const int c = seg * k, len = n - c < k ? n - c : k;
         if (c + len <= first) break;
         for (int j = 1; j <= len; ++j) {
-            pv::k_sweeps<T><<<n_tiles, sweep_block(), pv::sweep_smem_bytes<T>(), st>>>(
-                ddesc + (c + j - 1), nullptr, n_tiles, 1, 0, pv::GridSync{nullptr, nullptr, nullptr, 0});
+            launch_sweep<T>(ddesc + (c + j - 1), nullptr, n_tiles, 0, j, st);
             if ((s = launched(h)) != PIXVOD_OK) return s;
         }
         for (int j = len; j >= 1 && c + j > first; --j)
@@ -1335,8 +1357,7 @@ pixvod_status batch_sweeps(pixvod_batch* b, int n_iters, int schedule) {
         }
     } else if (schedule == PIXVOD_SCHED_BATCHED) {
         for (int it = 0; it < n_iters; ++it) {
-            pv::k_sweeps<T><<<b->n_work, sweep_block(), pv::sweep_smem_bytes<T>(), b->stream>>>(
-                descs<T>(b), works(b), b->n_work, 1, cur, pv::GridSync{nullptr, nullptr, nullptr, 0});
+            launch_sweep<T>(descs<T>(b), works(b), b->n_work, cur, cur, b->stream);
             if ((s = batch_launched(b)) != PIXVOD_OK) return s;
             cur ^= 1;
         }
@@ -1355,7 +1376,7 @@ pixvod_status batch_sweeps(pixvod_batch* b, int n_iters, int schedule) {
         const pv::SeqDesc<T>* d = descs<T>(b);
         const pv::Work* w = works(b);
         int n_work = b->n_work, cur0 = cur;
-        void* args[] = {(void*)&d, (void*)&w, (void*)&n_work, (void*)&n_iters, (void*)&cur0, (void*)&gs};
+        void* args[] = {(void*)&d, (void*)&w, (void*)&n_work, (void*)&n_iters, (void*)&cur0, (void*)&cur0, (void*)&gs};
         s = cuda_status(cudaLaunchCooperativeKernel((const void*)pv::k_sweeps<T>, dim3(grid), sweep_block(),
                                                     args, pv::sweep_smem_bytes<T>(), b->stream));
         b->launches++;

@@ -103,7 +103,8 @@ __device__ __forceinline__ bool grid_sync(const GridSync& gs) {
 template <typename T>
 __global__ void __launch_bounds__(SWEEP_THREADS, sizeof(T) == 4 ? 4 : 2) k_sweeps(const SeqDesc<T>* __restrict__ seqs,
                                                              const Work* __restrict__ work, int n_work,
-                                                             int n_iters, int cur0, GridSync gs) {
+                                                             int n_iters, int cur0, int flip0,
+                                                             GridSync gs) {
     // msg[p * TILE_PX + tid]: a tile's 108 identity-message planes, bulk-copied in
     // at the start of the tile (the old messages), overwritten in place by the
     // damped new ones
@@ -111,17 +112,24 @@ __global__ void __launch_bounds__(SWEEP_THREADS, sizeof(T) == 4 ? 4 : 2) k_sweep
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0 && threadIdx.y == 0) mbar_init(&bar, 1);
     __syncthreads();
+    pdl_wait();
     T* msg = reinterpret_cast<T*>(smem_raw);
     unsigned parity = 0;
     for (int it = 0; it < n_iters; ++it) {
         const int cur = (cur0 + it) & 1;
-        for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
+        // every other sweep takes the work from its end: what the previous sweep wrote
+        // last is what L2 still holds
+        const bool flip = (flip0 + it) & 1;
+        for (int k = blockIdx.x; k < n_work; k += gridDim.x) {
+            const int w = flip ? n_work - 1 - k : k;
             const Work wk = work ? work[w] : Work{0, w};
             const SweepArgs<T> a = seq_args(seqs[wk.seq], cur);
             // a tile whose bulk copy never arrived ends the block's work for the
             // launch: the mbarrier's phase no longer matches `parity`, and the copy
             // may still be writing `msg`
-            if (!sweep_tile(a, wk.tile % a.g.tiles_x, wk.tile / a.g.tiles_x, msg, &bar, parity)) return;
+            if (!sweep_tile(a, wk.tile % a.g.tiles_x, wk.tile / a.g.tiles_x, msg, &bar, parity,
+                            it + 1 == n_iters))
+                return;
             parity ^= 1u;
             if (n_iters > 1) asm volatile("fence.proxy.async.global;" ::: "memory");
             __syncthreads();

@@ -580,17 +580,30 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
     return true;
 }
 
-// shared -> global bulk copy by the calling thread, waited for until the writes
-// are complete and ordered before the thread's later generic-proxy accesses;
-// dst, src and bytes must be multiples of 16 bytes
-__device__ __forceinline__ void bulk_copy_s2g(void* dst, const void* src, unsigned bytes) {
+// shared -> global bulk copy by the calling thread; dst, src and bytes must be
+// multiples of 16 bytes. In a launch's last sweep only the reads of shared memory
+// are waited for (the end of the kernel completes the writes); before a grid
+// barrier, until the writes are complete and ordered before the thread's later
+// generic-proxy accesses.
+__device__ __forceinline__ void bulk_copy_s2g(void* dst, const void* src, unsigned bytes, bool last_sweep) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
                  "r"(bytes)
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-    asm volatile("fence.proxy.async.global;" ::: "memory");
+    if (last_sweep) {
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    } else {
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+    }
 }
+
+// Programmatic dependent launch: a kernel launched with the attribute may start
+// while its predecessor in the stream drains; pdl_wait returns when the
+// predecessor has completed and its writes are visible, pdl_trigger lets the
+// successor's blocks take the slots that this grid leaves free.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // One synchronous sweep over one state tile (tx, ty) by the calling block (every
 // thread of the block must call it). The block must have initialised `bar` (one
@@ -602,7 +615,7 @@ __device__ __forceinline__ void bulk_copy_s2g(void* dst, const void* src, unsign
 // block must take no further tile in this launch.
 template <typename T>
 __device__ __forceinline__ bool sweep_tile(const SweepArgs<T>& a, int tx, int ty, T* msg, uint64_t* bar,
-                                           unsigned parity) {
+                                           unsigned parity, bool last_sweep) {
     const int tid = threadIdx.y * SWEEP_BX + threadIdx.x;
     const size_t tile = (size_t)ty * a.g.tiles_x + tx;
     constexpr unsigned bytes = sizeof(T) * MSG_PLANES * TILE_PX;
@@ -619,7 +632,8 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs<T>& a, int tx, int ty
     // messages never arrived is not stored
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     const bool all_ok = __syncthreads_and(ok);
-    if (all_ok && tid == 0) bulk_copy_s2g(a.out + tile * TILE_WORDS + PL_ID * TILE_PX, msg, bytes);
+    if (last_sweep) pdl_trigger();
+    if (all_ok && tid == 0) bulk_copy_s2g(a.out + tile * TILE_WORDS + PL_ID * TILE_PX, msg, bytes, last_sweep);
     return all_ok;
 }
 
