@@ -40,7 +40,9 @@ constexpr int PL_ID = 35;
 constexpr int ID_STRIDE = 27;
 constexpr int PL_NM = 143;
 constexpr int N_INPUT_PLANES = 6;  // I_s, I_t, g_x, g_y, m_x, m_y (row-major, pitched)
-constexpr int MSG_PLANES = PL_NM - PL_ID;  // 108: the identity-message planes 35..142
+constexpr int MSG_PLANES = PL_NM - PL_ID;     // 108: the identity-message planes 35..142
+constexpr int LAM = 21;                       // planes of one message's Lambda
+constexpr int LAM_PLANES = 4 * LAM;           // staged through shared memory
 constexpr int TILE_W = 32;
 constexpr int TILE_H = 4;
 constexpr int TILE_PX = TILE_W * TILE_H;
@@ -111,6 +113,13 @@ struct SweepArgs {
 };
 
 
+// Programmatic dependent launch: a kernel launched with the attribute may start
+// while its predecessor in the stream drains; pdl_wait returns when the
+// predecessor has completed and its writes are visible, pdl_trigger lets the
+// successor's blocks take the slots that this grid leaves free.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
 // a0: frame ingest
 // ---------------------------------------------------------------------------
@@ -153,6 +162,7 @@ __device__ __forceinline__ void ingest_keyframe_px(const Geometry<T>& g, const f
 template <typename T>
 __global__ void k_ingest_keyframe(Geometry<T> g, const float* __restrict__ frame,
                                   const float* __restrict__ normals, T* I_s, T* m_x, T* m_y) {
+    pdl_wait();
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     int v = blockIdx.y * blockDim.y + threadIdx.y;
     if (u >= g.W || v >= g.H) return;
@@ -174,6 +184,7 @@ __device__ __forceinline__ void ingest_target_px(const Geometry<T>& g, const flo
 
 template <typename T>
 __global__ void k_ingest_target(Geometry<T> g, const float* __restrict__ frame, T* I_t, T* g_x, T* g_y) {
+    pdl_wait();
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     int v = blockIdx.y * blockDim.y + threadIdx.y;
     if (u >= g.W || v >= g.H) return;
@@ -208,6 +219,7 @@ __global__ void k_poison_outside(Geometry<T> g, int n_tiles, T* state) {
 
 template <typename T>
 __global__ void k_reset(Geometry<T> g, Factors<T> f, T* state, const Scalars* sc) {
+    pdl_wait();
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     int v = blockIdx.y * blockDim.y + threadIdx.y;
     if (u >= g.W || v >= g.H) return;
@@ -272,24 +284,34 @@ __device__ __forceinline__ T ld_state(const T* p) {
 }
 
 // Thread block of the sweep kernel: one state tile (32 x 4 pixels), one thread
-// per pixel; 4 blocks per SM (55 KB of shared memory and at most 128 registers
-// each). Each thread keeps its four damped identity messages in shared memory
-// until the belief solve has given tau; their eta is then projected in place and
-// the tile's 108 message planes leave with one bulk copy. The identity-message
-// loop is not unrolled; the normal messages are computed in a loop of their own
-// after it and stay in registers.
+// per pixel; 4 blocks per SM (43 KB of shared memory and at most 128 registers
+// each). What a tile waits on is memory latency (at 640x480 about 34 of the 46
+// thousand clocks that it took; no pipe or bandwidth above 45 %), so loads are
+// issued early and together and the register file holds as many pixels as it can:
+//  - the four messages' Lambda are bulk-copied into shared memory, damped in place
+//    and bulk-copied out; M_p is summed from there after the loop instead of in 21
+//    registers through it. Their eta (24 of 108 planes) go straight to and from
+//    global memory: the old ones load with the neighbour's values, the new ones
+//    come back for the tangent projection under the mean update's arithmetic.
+//    (All 108 planes staged, M_p in registers: 89.1 against 86.4 us per sweep at
+//    640x480, 850 against 814 us at 2048x1536.)
+//  - the photometric factor comes first, its taps loading under the bulk copy
+//    (after the loop: 90.9 against 89.1 us, 886 against 850 us).
+// Five blocks per SM at 96 registers were slower (96.1 us, 936 us): the spills and
+// a larger working set in L2 cost more than the extra warps hide. The identity
+// loop is not unrolled; the normal messages are computed in a loop of their own.
 constexpr int SWEEP_BX = TILE_W;
 constexpr int SWEEP_BY = TILE_H;
 constexpr int SWEEP_THREADS = TILE_PX;
 
 template <typename T>
 constexpr size_t sweep_smem_bytes() {
-    return sizeof(T) * MSG_PLANES * TILE_PX;
+    return sizeof(T) * LAM_PLANES * TILE_PX;
 }
 
 // The calling thread's pixel of the sweep over tile (tx, ty): everything but the
-// store of the identity messages, which are left, projected, in `msg`. False if
-// the tile's bulk copy never arrived (FLAG_TIMEOUT is set).
+// store of the identity messages' Lambda, which are left in `msg`. False if the
+// tile's bulk copy never arrived (FLAG_TIMEOUT is set).
 template <typename T>
 __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int ty, T* msg, uint64_t* bar,
                                             unsigned parity) {
@@ -325,99 +347,10 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
 #pragma unroll
     for (int q = 0; q < 7; ++q) eb[q] = T(0);
     // --- priors (Eq. 4 with identity Jacobian; log-depth prior) ---
-    T Mp[21];
 #pragma unroll
-    for (int q = 0; q < 21; ++q) Mp[q] = T(0);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        Mp[pidx(k, k)] = F.lam_P;
-        eb[k] -= F.lam_P * xi[k];
-    }
+    for (int k = 0; k < 6; ++k) eb[k] -= F.lam_P * xi[k];
     T md = F.lam_Z;
     eb[6] -= F.lam_Z * (d - T(a.sc->d_prior));
-
-    // --- a2/a3: pairwise messages from the four neighbours ---
-    if (!mbar_wait_bounded(bar, parity)) {
-        // the tile's messages never arrived: flag it, wait once more, leave the tile
-        atomicOr(&a.sc->flags, FLAG_TIMEOUT);
-        mbar_wait_bounded(bar, parity);
-        return false;
-    }
-    const T beta = F.beta, omb = T(1) - F.beta;
-#pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
-        T* mb = msg + PV_IDX((k * ID_STRIDE) * TILE_PX + tid, (MSG_PLANES - ID_STRIDE + 1) * TILE_PX, flags);  // slot k
-        const int un = u + (k == 0 ? -1 : (k == 1 ? 1 : 0));
-        const int vn = v + (k == 2 ? -1 : (k == 3 ? 1 : 0));
-        const bool has = un >= 0 && un < g.W && vn >= 0 && vn < g.H;
-        if (!has) {
-#pragma unroll
-            for (int q = 0; q < ID_STRIDE; ++q) mb[q * TILE_PX] = T(0);
-            continue;
-        }
-        const int ko = k ^ 1;
-        const T* Sj = a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags);
-        // variable-to-factor marginal of j: V = W + u u^T with W = M_p,j - Lambda_{f->j}
-        // (pose prior plus j's three other identity messages) and u = u_j, and
-        // eta_v = -eta_{f->j}. All of j's loads are issued here, ahead of the Exp/Log
-        // chain of the residual, so that their latency overlaps it.
-        const T* mj = Sj + (PL_ID + ID_STRIDE * ko) * TILE_PX;
-        T W[21], uj[6], gv[6], xj[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) xj[q] = ld_state(Sj + q * TILE_PX);
-#pragma unroll
-        for (int q = 0; q < 21; ++q) W[q] = ld_state(Sj + (PL_MP + q) * TILE_PX) - ld_state(mj + q * TILE_PX);
-#pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            uj[q] = ld_state(Sj + (PL_U + q) * TILE_PX);
-            gv[q] = -ld_state(mj + (21 + q) * TILE_PX);
-        }
-        T rb[6];
-        se3_between(xj, qi, t, rb);
-        IdMsg<T> m;
-        if (!identity_msg(W, uj, gv, rb, F.lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
-        // damped: (1 - beta) new + beta old, over the old message in shared memory
-        const T wl = omb * F.lam_R, wll = wl * F.lam_R;
-#pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            const T e = v_fma(wl, m.he[q], beta * mb[(21 + q) * TILE_PX]);
-            eb[q] += e;
-            mb[(21 + q) * TILE_PX] = e;
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c)
-#pragma unroll
-            for (int r = c; r < 6; ++r) {
-                const T l = m.lambda(r, c, wl, wll, beta * mb[pidx(r, c) * TILE_PX]);
-                Mp[pidx(r, c)] += l;
-                mb[pidx(r, c) * TILE_PX] = l;
-            }
-    }
-
-    // normal-integration factors (Eq. 6): r_i = d_i - d_j + sg m
-    T nl[4], ne[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        nl[k] = T(0);
-        ne[k] = T(0);
-        const int un = u + (k == 0 ? -1 : (k == 1 ? 1 : 0));
-        const int vn = v + (k == 2 ? -1 : (k == 3 ? 1 : 0));
-        if (!(un >= 0 && un < g.W && vn >= 0 && vn < g.H)) continue;
-        const int ko = k ^ 1;
-        const T* Sj = a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags);
-        T dj = ld_state(Sj + 6 * TILE_PX);
-        T sv = ld_state(Sj + PL_S * TILE_PX) - ld_state(Sj + (PL_NM + 2 * ko) * TILE_PX);
-        T evn = -ld_state(Sj + (PL_NM + 2 * ko + 1) * TILE_PX);
-        T m = k == 0 ? a.m_x[PV_IDX(i - 1, n_plane, flags)]
-                     : (k == 1 ? a.m_x[i] : (k == 2 ? a.m_y[PV_IDX(i - g.pitch, n_plane, flags)] : a.m_y[i]));
-        T sg = (k == 0 || k == 2) ? T(1) : T(-1);
-        T rn = d - dj + sg * m;
-        T den = v_div(T(1), F.lam_N + sv);
-        nl[k] = omb * (F.lam_N * sv * den) + beta * ld_state(Si + (PL_NM + 2 * k) * TILE_PX);
-        ne[k] = omb * (F.lam_N * (evn - sv * rn) * den) + beta * ld_state(Si + (PL_NM + 2 * k + 1) * TILE_PX);
-        md += nl[k];
-        eb[6] += ne[k];
-    }
 
     T alpha = T(0), rph = T(0);
     T J[7];
@@ -488,6 +421,106 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
             br = hub ? (BR_VALID | BR_HUBER) : BR_VALID;
         }
     }
+    // --- a2/a3: pairwise messages from the four neighbours ---
+    if (!mbar_wait_bounded(bar, parity)) {
+        // the tile's messages never arrived: flag it, wait once more, leave the tile
+        atomicOr(&a.sc->flags, FLAG_TIMEOUT);
+        mbar_wait_bounded(bar, parity);
+        return false;
+    }
+    const T beta = F.beta, omb = T(1) - F.beta;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        T* mb = msg + PV_IDX((k * LAM) * TILE_PX + tid, (LAM_PLANES - LAM + 1) * TILE_PX, flags);  // slot k
+        T* me = Di + (PL_ID + ID_STRIDE * k + LAM) * TILE_PX;                                                    // its eta
+        const int un = u + (k == 0 ? -1 : (k == 1 ? 1 : 0));
+        const int vn = v + (k == 2 ? -1 : (k == 3 ? 1 : 0));
+        const bool has = un >= 0 && un < g.W && vn >= 0 && vn < g.H;
+        if (!has) {
+#pragma unroll
+            for (int q = 0; q < 21; ++q) mb[q * TILE_PX] = T(0);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) me[q * TILE_PX] = T(0);
+            continue;
+        }
+        const int ko = k ^ 1;
+        const T* Sj = a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags);
+        // variable-to-factor marginal of j: V = W + u u^T with W = M_p,j - Lambda_{f->j}
+        // (pose prior plus j's three other identity messages) and u = u_j, and
+        // eta_v = -eta_{f->j}. All of j's loads are issued here, ahead of the Exp/Log
+        // chain of the residual, so that their latency overlaps it.
+        const T* mj = Sj + (PL_ID + ID_STRIDE * ko) * TILE_PX;
+        T W[21], uj[6], gv[6], xj[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) xj[q] = ld_state(Sj + q * TILE_PX);
+#pragma unroll
+        for (int q = 0; q < 21; ++q) W[q] = ld_state(Sj + (PL_MP + q) * TILE_PX) - ld_state(mj + q * TILE_PX);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            uj[q] = ld_state(Sj + (PL_U + q) * TILE_PX);
+            gv[q] = -ld_state(mj + (21 + q) * TILE_PX);
+        }
+        T eo[6];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) eo[q] = ld_state(Si + (PL_ID + ID_STRIDE * k + LAM + q) * TILE_PX);
+        T rb[6];
+        se3_between(xj, qi, t, rb);
+        IdMsg<T> m;
+        if (!identity_msg(W, uj, gv, rb, F.lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
+        // damped: (1 - beta) new + beta old; Lambda over the old one in shared memory
+        const T wl = omb * F.lam_R, wll = wl * F.lam_R;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const T e = v_fma(wl, m.he[q], beta * eo[q]);
+            eb[q] += e;
+            me[q * TILE_PX] = e;
+        }
+#pragma unroll
+        for (int c = 0; c < 6; ++c)
+#pragma unroll
+            for (int r = c; r < 6; ++r) {
+                const T l = m.lambda(r, c, wl, wll, beta * mb[pidx(r, c) * TILE_PX]);
+                mb[pidx(r, c) * TILE_PX] = l;
+            }
+    }
+    // M_p from the four messages in shared memory
+    T Mp[21];
+#pragma unroll
+    for (int q = 0; q < 21; ++q) {
+        T x = T(0);
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (q == pidx(k, k)) x = F.lam_P;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x += msg[(LAM * k + q) * TILE_PX + tid];
+        Mp[q] = x;
+    }
+
+    // normal-integration factors (Eq. 6): r_i = d_i - d_j + sg m
+    T nl[4], ne[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        nl[k] = T(0);
+        ne[k] = T(0);
+        const int un = u + (k == 0 ? -1 : (k == 1 ? 1 : 0));
+        const int vn = v + (k == 2 ? -1 : (k == 3 ? 1 : 0));
+        if (!(un >= 0 && un < g.W && vn >= 0 && vn < g.H)) continue;
+        const int ko = k ^ 1;
+        const T* Sj = a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags);
+        T dj = ld_state(Sj + 6 * TILE_PX);
+        T sv = ld_state(Sj + PL_S * TILE_PX) - ld_state(Sj + (PL_NM + 2 * ko) * TILE_PX);
+        T evn = -ld_state(Sj + (PL_NM + 2 * ko + 1) * TILE_PX);
+        T m = k == 0 ? a.m_x[PV_IDX(i - 1, n_plane, flags)]
+                     : (k == 1 ? a.m_x[i] : (k == 2 ? a.m_y[PV_IDX(i - g.pitch, n_plane, flags)] : a.m_y[i]));
+        T sg = (k == 0 || k == 2) ? T(1) : T(-1);
+        T rn = d - dj + sg * m;
+        T den = v_div(T(1), F.lam_N + sv);
+        nl[k] = omb * (F.lam_N * sv * den) + beta * ld_state(Si + (PL_NM + 2 * k) * TILE_PX);
+        ne[k] = omb * (F.lam_N * (evn - sv * rn) * den) + beta * ld_state(Si + (PL_NM + 2 * k + 1) * TILE_PX);
+        md += nl[k];
+        eb[6] += ne[k];
+    }
+
     // --- a4: belief, mean update, tangent projection ---
     // With B = blockdiag(M_p, m_d), h = B^-1 eta_o and z = B^-1 J, Sherman-Morrison
     // gives tau = Lambda_b^-1 eta_b = h - z alpha (r + J^T h) / (1 + alpha J^T z),
@@ -539,6 +572,12 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
         for (int q = 0; q < 7; ++q) tau[q] = T(0);
     }
     if (a.br) a.br[tile * TILE_PX + tid] = br;
+    // the new eta, back for the projection below
+    T en[24];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int q = 0; q < 6; ++q) en[6 * k + q] = __ldcg(Di + (PL_ID + ID_STRIDE * k + LAM + q) * TILE_PX);
     // mu <- mu (+) tau
     {
         T xn[6];
@@ -562,33 +601,33 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
         Di[(PL_NM + 2 * k) * TILE_PX] = nl[k];
         Di[(PL_NM + 2 * k + 1) * TILE_PX] = ne[k] - nl[k] * tau[6];
     }
-#pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
-        T* mb = msg + (k * ID_STRIDE) * TILE_PX + tid;
-        T L[21];
 #pragma unroll
-        for (int q = 0; q < 21; ++q) L[q] = mb[q * TILE_PX];
+    for (int k = 0; k < 4; ++k) {
+        const T* mb = msg + (k * LAM) * TILE_PX + tid;
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
-            T e = mb[(21 + r) * TILE_PX];
+            T e = en[6 * k + r];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) e -= L[pidx(r, c)] * tau[c];
-            mb[(21 + r) * TILE_PX] = e;
+            for (int c = 0; c < 6; ++c) e -= mb[pidx(r, c) * TILE_PX] * tau[c];
+            Di[(PL_ID + ID_STRIDE * k + LAM + r) * TILE_PX] = e;
         }
     }
     if (flags) atomicOr(&a.sc->flags, flags);
     return true;
 }
 
-// shared -> global bulk copy by the calling thread; dst, src and bytes must be
-// multiples of 16 bytes. In a launch's last sweep only the reads of shared memory
-// are waited for (the end of the kernel completes the writes); before a grid
-// barrier, until the writes are complete and ordered before the thread's later
-// generic-proxy accesses.
-__device__ __forceinline__ void bulk_copy_s2g(void* dst, const void* src, unsigned bytes, bool last_sweep) {
+// shared -> global bulk copy by the calling thread, part of its current bulk
+// group; dst, src and bytes must be multiples of 16 bytes
+__device__ __forceinline__ void bulk_copy_s2g(void* dst, const void* src, unsigned bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)),
                  "r"(bytes)
                  : "memory");
+}
+// Wait for the group. In a launch's last sweep only the reads of shared memory are
+// waited for (the end of the kernel completes the writes); before a grid barrier,
+// until the writes are complete and ordered before the thread's later
+// generic-proxy accesses.
+__device__ __forceinline__ void bulk_wait_s2g(bool last_sweep) {
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     if (last_sweep) {
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -598,18 +637,11 @@ __device__ __forceinline__ void bulk_copy_s2g(void* dst, const void* src, unsign
     }
 }
 
-// Programmatic dependent launch: a kernel launched with the attribute may start
-// while its predecessor in the stream drains; pdl_wait returns when the
-// predecessor has completed and its writes are visible, pdl_trigger lets the
-// successor's blocks take the slots that this grid leaves free.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // One synchronous sweep over one state tile (tx, ty) by the calling block (every
 // thread of the block must call it). The block must have initialised `bar` (one
 // arrival); `parity` is the phase this tile's bulk copy completes. The caller
 // synchronises the block before reusing `msg` for another tile. The message
-// planes of pixels outside the image are copied through unchanged. Returns
+// Lambda planes of pixels outside the image are copied through unchanged. Returns
 // false (to every thread) when the tile's bulk copy did not arrive within the
 // bounded wait: nothing of the tile was stored, FLAG_TIMEOUT is set, and the
 // block must take no further tile in this launch.
@@ -618,22 +650,28 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs<T>& a, int tx, int ty
                                            unsigned parity, bool last_sweep) {
     const int tid = threadIdx.y * SWEEP_BX + threadIdx.x;
     const size_t tile = (size_t)ty * a.g.tiles_x + tx;
-    constexpr unsigned bytes = sizeof(T) * MSG_PLANES * TILE_PX;
+    constexpr unsigned bytes = sizeof(T) * LAM * TILE_PX;  // one message's Lambda planes
     if (tid == 0) {
         // order earlier generic-proxy accesses (global stores of a previous sweep in
         // the same launch, shared-memory use of a previous tile) before the async copy
         asm volatile("fence.proxy.async;" ::: "memory");
-        mbar_expect_tx(bar, bytes);
-        bulk_copy_g2s(msg, a.in + tile * TILE_WORDS + PL_ID * TILE_PX, bytes, bar);
+        mbar_expect_tx(bar, 4 * bytes);
+        for (int k = 0; k < 4; ++k)
+            bulk_copy_g2s(msg + LAM * k * TILE_PX, a.in + tile * TILE_WORDS + (PL_ID + ID_STRIDE * k) * TILE_PX, bytes,
+                          bar);
     }
     const bool ok = sweep_pixel(a, tx, ty, msg, bar, parity);
-    // the projected messages written to shared memory (generic proxy) are read by
+    // the messages written to shared memory (generic proxy) are read by
     // the bulk copy (async proxy): fence, then gather the block; a tile whose
     // messages never arrived is not stored
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     const bool all_ok = __syncthreads_and(ok);
     if (last_sweep) pdl_trigger();
-    if (all_ok && tid == 0) bulk_copy_s2g(a.out + tile * TILE_WORDS + PL_ID * TILE_PX, msg, bytes, last_sweep);
+    if (all_ok && tid == 0) {
+        for (int k = 0; k < 4; ++k)
+            bulk_copy_s2g(a.out + tile * TILE_WORDS + (PL_ID + ID_STRIDE * k) * TILE_PX, msg + LAM * k * TILE_PX, bytes);
+        bulk_wait_s2g(last_sweep);
+    }
     return all_ok;
 }
 
@@ -641,6 +679,27 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs<T>& a, int tx, int ty
 // a5: pose average (App. C.2) and keyframe anchoring, one launch, fixed order
 // ---------------------------------------------------------------------------
 constexpr int RED_THREADS = TILE_PX;
+
+// Seven sums over the block's threads, in a fixed order (shuffles within a warp,
+// then the warps in order), in every thread of warp 0; one barrier where a
+// shared-memory tree took seven.
+__device__ __forceinline__ void block_sum7(double* r, double (*sh)[RED_THREADS / 32]) {
+    __syncthreads();  // sh may still be read from an earlier sum
+#pragma unroll
+    for (int q = 0; q < 7; ++q)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r[q] += __shfl_xor_sync(0xffffffffu, r[q], o);
+    if ((threadIdx.x & 31) == 0)
+#pragma unroll
+        for (int q = 0; q < 7; ++q) sh[q][threadIdx.x >> 5] = r[q];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+        r[q] = sh[q][0];
+#pragma unroll
+        for (int w = 1; w < RED_THREADS / 32; ++w) r[q] += sh[q][w];
+    }
+}
 
 // One block per state tile sums that tile's 7 mean planes (double accumulation,
 // fixed order); the last block to finish sums the tile partials in tile order,
@@ -650,55 +709,41 @@ template <typename T>
 __device__ __forceinline__ void reduce_tile(const Geometry<T>& g, const T* __restrict__ state,
                                             double* __restrict__ partials, Scalars* sc, int anchor, int tile,
                                             int n_tiles) {
-    __shared__ double sh[7][RED_THREADS];
+    __shared__ double sh[7][RED_THREADS / 32];
     __shared__ bool last;
     const int tid = threadIdx.x;
     const int u = (tile % g.tiles_x) * TILE_W + tid % TILE_W;
     const int v = (tile / g.tiles_x) * TILE_H + tid / TILE_W;
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    if (tid < TILE_PX && u < g.W && v < g.H) {
+    double r[7] = {0, 0, 0, 0, 0, 0, 0};
+    if (u < g.W && v < g.H) {
         const T* st = state + (size_t)tile * TILE_WORDS + tid;
 #pragma unroll
-        for (int q = 0; q < 7; ++q) acc[q] = double(st[q * TILE_PX]);
+        for (int q = 0; q < 7; ++q) r[q] = double(st[q * TILE_PX]);
     }
-#pragma unroll
-    for (int q = 0; q < 7; ++q) sh[q][tid] = acc[q];
-    __syncthreads();
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if (tid < s)
-#pragma unroll
-            for (int q = 0; q < 7; ++q) sh[q][tid] += sh[q][tid + s];
-        __syncthreads();
-    }
+    block_sum7(r, sh);
     if (tid == 0) {
 #pragma unroll
-        for (int q = 0; q < 7; ++q) partials[tile * 7 + q] = sh[q][0];
+        for (int q = 0; q < 7; ++q) partials[tile * 7 + q] = r[q];
         __threadfence();
         last = atomicAdd(&sc->counter, 1u) == (unsigned)(n_tiles - 1);
     }
     __syncthreads();
     if (!last) return;
-    double r[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < 7; ++q) r[q] = 0.0;
+#pragma unroll 4
     for (int h = tid; h < n_tiles; h += RED_THREADS)
 #pragma unroll
         for (int q = 0; q < 7; ++q) r[q] += __ldcg(partials + h * 7 + q);
-#pragma unroll
-    for (int q = 0; q < 7; ++q) sh[q][tid] = r[q];
-    __syncthreads();
-    for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
-        if (tid < s)
-#pragma unroll
-            for (int q = 0; q < 7; ++q) sh[q][tid] += sh[q][tid + s];
-        __syncthreads();
-    }
+    block_sum7(r, sh);
     if (tid == 0) {
         const double n = double(g.W) * double(g.H);
         double xi[6], R[9], t[3];
         for (int q = 0; q < 6; ++q) {
-            xi[q] = sh[q][0] / n;
+            xi[q] = r[q] / n;
             sc->xi_est[q] = xi[q];
         }
-        sc->d_mean = sh[6][0] / n;
+        sc->d_mean = r[6] / n;
         se3_exp(xi, R, t);
         // T_cur = Exp(xi_est) T_kf with Exp(xi_est) = [R t; 0 1]
         double Tc[16];
@@ -721,12 +766,14 @@ template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce(Geometry<T> g, const T* __restrict__ state,
                                                         double* __restrict__ partials, Scalars* sc,
                                                         int anchor) {
+    pdl_wait();
     reduce_tile(g, state, partials, sc, anchor, blockIdx.x, gridDim.x);
 }
 
 // Depth output: exp(sign * mu_6) as dense float32.
 template <typename T>
 __global__ void k_depth_out(Geometry<T> g, const T* __restrict__ state, float* out, T sign) {
+    pdl_wait();
     int u = blockIdx.x * blockDim.x + threadIdx.x;
     int v = blockIdx.y * blockDim.y + threadIdx.y;
     if (u >= g.W || v >= g.H) return;
