@@ -56,10 +56,10 @@ struct Layout {
     size_t total;
 };
 
-// the quadtree region at off_qt: two QtArgs (room for FP64), then the three
+// the quadtree region at off_qt: two QtArgs (room for FP64), then the two
 // kernels' block offsets {0, blocks}
 constexpr size_t kQtArgsBytes = 2 * sizeof(pv::QtArgs<double>);
-constexpr size_t kQtRegionBytes = kQtArgsBytes + 6 * sizeof(int);
+constexpr size_t kQtRegionBytes = kQtArgsBytes + 4 * sizeof(int);
 
 bool intrinsics_ok(const pixvod_intrinsics* K) {
     return K && K->width >= 2 && K->height >= 2 && K->width <= 32768 && K->height <= 32768 &&
@@ -219,6 +219,7 @@ struct pixvod_handle {
     int rec_n;           // sweeps of the recorded frame (0: none)
     int rec_window;      // differentiate only the last rec_window sweeps (0: all)
     bool rec_valid;      // the recorded frame can be differentiated
+    bool qt_stale;       // quadtree: the loaded state has values in identity slots 1..3
     // profiling
     bool profiling;
     std::vector<cudaEvent_t> ev;
@@ -417,19 +418,21 @@ pv::QtArgs<T> qt_args(pixvod_handle* h) {
     return a;
 }
 
-// blocks of 128 threads of k_qt_node_msgs: one thread per pixel (tile order),
-// per child slot of the nodes of levels >= 2 (each slot's run padded to a warp),
-// and per node's parent slot
-unsigned qt_msg_blocks(const pixvod_handle* h) {
+// blocks of the quadtree sweep's two kernels. k_qt_messages: one per 32 x 4 pixels,
+// then, per 128 node messages, a thread per pixel (tile order), per child slot of
+// the nodes of levels >= 2 (each slot's run padded to a warp) and per node's parent
+// slot; k_qt_node_belief: one per 128 nodes
+int qt_message_blocks(const pixvod_handle* h) {
     const pv::QtGeom& q = h->L.q;
     const size_t n_px = (size_t)h->L.tiles_x * h->L.tiles_y * pv::TILE_PX;
     const size_t n_up = q.n_levels > 1 ? (size_t)(q.n_nodes - q.base[1]) : 0;
     const size_t threads = n_px + 4 * ((n_up + 31) / 32 * 32) + (size_t)q.n_nodes;
-    return (unsigned)((threads + 127) / 128);
+    return h->L.tiles_x * h->L.tiles_y + (int)((threads + 127) / 128);
 }
+int qt_belief_blocks(const pixvod_handle* h) { return (h->L.q.n_nodes + 127) / 128; }
 
 // a quadtree handle's sweep arguments in its workspace, for cur = 0 and 1, and
-// the three kernels' block offsets {0, blocks}: a batch of one sequence, so that
+// the two kernels' block offsets {0, blocks}: a batch of one sequence, so that
 // a handle and a batch run the same kernels. Written once (pointers into the
 // workspace, geometry, factor weights).
 template <typename T>
@@ -441,8 +444,7 @@ pixvod_status upload_qt_handle(pixvod_handle* h) {
         args[c] = qt_args<T>(h);
     }
     h->cur = keep;
-    const dim3 pg = pixel_grid(h);
-    const int off[6] = {0, (int)(pg.x * pg.y), 0, (int)qt_msg_blocks(h), 0, (h->L.q.n_nodes + 127) / 128};
+    const int off[4] = {0, qt_message_blocks(h), 0, qt_belief_blocks(h)};
     pixvod_status s = cuda_status(
         cudaMemcpyAsync(h->ws + h->L.off_qt, args, sizeof(args), cudaMemcpyHostToDevice, h->stream));
     if (s == PIXVOD_OK)
@@ -457,14 +459,17 @@ template <typename T>
 pixvod_status launch_qt_sweep(pixvod_handle* h) {
     const pv::QtArgs<T>* A = reinterpret_cast<const pv::QtArgs<T>*>(h->ws + h->L.off_qt) + h->cur;
     const int* off = reinterpret_cast<const int*>(h->ws + h->L.off_qt + kQtArgsBytes);
-    const dim3 pg = pixel_grid(h);
-    pv::k_qt_pixels<T><<<pg.x * pg.y, pixel_block(), 0, h->stream>>>(A, off, 1);
+    launch_pdl(pv::k_qt_messages<T>, dim3(qt_message_blocks(h)), pixel_block(), 0, h->stream, A, off, 1);
     pixvod_status s = launched(h);
     if (s != PIXVOD_OK) return s;
-    pv::k_qt_node_msgs<T><<<qt_msg_blocks(h), 128, 0, h->stream>>>(A, off + 2, 1);
-    if ((s = launched(h)) != PIXVOD_OK) return s;
-    pv::k_qt_node_belief<T><<<(h->L.q.n_nodes + 127) / 128, 128, 0, h->stream>>>(A, off + 4, 1);
-    return launched(h);
+    launch_pdl(pv::k_qt_node_belief<T>, dim3(qt_belief_blocks(h)), dim3(128), 0, h->stream, A, off + 2, 1);
+    if ((s = launched(h)) != PIXVOD_OK || !h->qt_stale) return s;
+    // a loaded checkpoint's unused identity slots, now consumed: zero from here on
+    h->qt_stale = false;
+    return cuda_status(cudaMemset2DAsync(state_ptr<T>(h, h->cur) + (pv::PL_ID + pv::ID_STRIDE) * pv::TILE_PX,
+                                         pv::TILE_WORDS * sizeof(T), 0,
+                                         (pv::MSG_PLANES - pv::ID_STRIDE) * pv::TILE_PX * sizeof(T),
+                                         (size_t)h->L.tiles_x * h->L.tiles_y, h->stream));
 }
 
 template <typename T>
@@ -551,20 +556,20 @@ pixvod_status run_sweeps_recorded(pixvod_handle* h, int n) {
 
 template <typename T>
 pixvod_status run_reduce(pixvod_handle* h, int anchor) {
-    pv::k_reduce<T><<<h->L.tiles_x * h->L.tiles_y, pv::RED_THREADS, 0, h->stream>>>(
-        geometry<T>(h), state_ptr<T>(h, h->cur), reinterpret_cast<double*>(h->ws + h->L.off_partials),
-        scalars(h), anchor);
+    launch_pdl(pv::k_reduce<T>, dim3(h->L.tiles_x * h->L.tiles_y), dim3(pv::RED_THREADS), 0, h->stream,
+               geometry<T>(h), state_ptr<T>(h, h->cur), reinterpret_cast<double*>(h->ws + h->L.off_partials),
+               scalars(h), anchor);
     return launched(h);
 }
 
 template <typename T>
 pixvod_status set_keyframe(pixvod_handle* h, const float* d_frame, const float* d_normals) {
-    pv::k_ingest_keyframe<T><<<pixel_grid(h), pixel_block(), 0, h->stream>>>(
-        geometry<T>(h), d_frame, d_normals, input_ptr<T>(h, 0), input_ptr<T>(h, 4), input_ptr<T>(h, 5));
+    launch_pdl(pv::k_ingest_keyframe<T>, pixel_grid(h), pixel_block(), 0, h->stream, geometry<T>(h), d_frame,
+               d_normals, input_ptr<T>(h, 0), input_ptr<T>(h, 4), input_ptr<T>(h, 5));
     pixvod_status s = launched(h);
     if (s != PIXVOD_OK) return s;
-    pv::k_reset<T><<<pixel_grid(h), pixel_block(), 0, h->stream>>>(geometry<T>(h), factors<T>(h),
-                                                                    state_ptr<T>(h, h->cur), scalars(h));
+    launch_pdl(pv::k_reset<T>, pixel_grid(h), pixel_block(), 0, h->stream, geometry<T>(h), factors<T>(h),
+               state_ptr<T>(h, h->cur), scalars(h));
     s = launched(h);
     if (s != PIXVOD_OK || !is_quadtree(h)) return s;
     pv::k_qt_reset<T><<<(h->L.q.n_nodes + 127) / 128, 128, 0, h->stream>>>(h->L.q, factors<T>(h).lam_P,
@@ -586,8 +591,8 @@ pixvod_status track_impl(pixvod_handle* h, const float* d_frame, const float* d_
     const bool kf = h->p.kf_interval > 0 && h->frame_index % h->p.kf_interval == 0;
     if (h->rec_ws && n_iters > h->RL.max_iters) return PIXVOD_EINVAL;
     h->rec_valid = false;
-    pv::k_ingest_target<T><<<pixel_grid(h), pixel_block(), 0, h->stream>>>(
-        geometry<T>(h), d_frame, input_ptr<T>(h, 1), input_ptr<T>(h, 2), input_ptr<T>(h, 3));
+    launch_pdl(pv::k_ingest_target<T>, pixel_grid(h), pixel_block(), 0, h->stream, geometry<T>(h), d_frame,
+               input_ptr<T>(h, 1), input_ptr<T>(h, 2), input_ptr<T>(h, 3));
     if ((s = launched(h)) != PIXVOD_OK) return s;
     if (h->rec_ws) {
         if ((s = run_sweeps_recorded<T>(h, n_iters)) != PIXVOD_OK) return s;
@@ -884,6 +889,7 @@ pixvod_status pixvod_create(const pixvod_intrinsics* K, const pixvod_params* p, 
     h->rec_n = 0;
     h->rec_window = 0;
     h->rec_valid = false;
+    h->qt_stale = false;
     pixvod_status s = cuda_status(cudaMemsetAsync(h->ws, 0, L.total, h->stream));
     if (s == PIXVOD_OK) {
         // T_kf = T_cur = identity
@@ -981,11 +987,11 @@ pixvod_status pixvod_get_pose_device(pixvod_handle* h, double* d_xi) {
 static pixvod_status depth_out(pixvod_handle* h, float* d_out, double sign) {
     if (!h || !d_out || !aligned(d_out, 4)) return PIXVOD_EINVAL;
     if (h->p.precision == 64)
-        pv::k_depth_out<double><<<pixel_grid(h), pixel_block(), 0, h->stream>>>(
-            geometry<double>(h), state_ptr<double>(h, h->cur), d_out, sign);
+        launch_pdl(pv::k_depth_out<double>, pixel_grid(h), pixel_block(), 0, h->stream, geometry<double>(h),
+                   state_ptr<double>(h, h->cur), d_out, sign);
     else
-        pv::k_depth_out<float><<<pixel_grid(h), pixel_block(), 0, h->stream>>>(
-            geometry<float>(h), state_ptr<float>(h, h->cur), d_out, float(sign));
+        launch_pdl(pv::k_depth_out<float>, pixel_grid(h), pixel_block(), 0, h->stream, geometry<float>(h),
+                   state_ptr<float>(h, h->cur), d_out, float(sign));
     return launched(h);
 }
 
@@ -1091,6 +1097,11 @@ pixvod_status pixvod_load_state(pixvod_handle* h, const void* h_buf, size_t byte
     if ((s = cuda_status(cudaStreamSynchronize(h->stream))) != PIXVOD_OK) return s;
     h->frame_index = hd[7];
     h->has_target = hd[11] == 1;
+    if (is_quadtree(h)) {  // identity slots 1..3 are zero in every state but a foreign one
+        const size_t lo = kHeaderBytes + pb * (pv::PL_ID + pv::ID_STRIDE), hi = kHeaderBytes + pb * pv::PL_NM;
+        h->qt_stale = false;
+        for (size_t k = lo; k < hi && !h->qt_stale; ++k) h->qt_stale = buf[k] != 0;
+    }
     return PIXVOD_OK;
 }
 
@@ -1231,11 +1242,11 @@ struct pixvod_batch {
     int64_t frame_index;
     int64_t launches;
     // quadtree sequences: the batched sweep's arguments (QtArgs<T> of every
-    // sequence for cur = 0, then for cur = 1) and, per kernel (pixels, node
-    // messages, node beliefs), the prefix sums of blocks per sequence
+    // sequence for cur = 0, then for cur = 1) and, per kernel (messages, node
+    // beliefs), the prefix sums of blocks per sequence
     bool qt;
     size_t off_qtargs, off_qtoff;
-    int qt_blocks[3];
+    int qt_blocks[2];
 };
 
 namespace {
@@ -1267,7 +1278,7 @@ BatchLayout make_batch_layout(int n, const pixvod_intrinsics* K, const pixvod_pa
     if (p->topology == PIXVOD_TOPOLOGY_QUADTREE) {
         off += align_up((size_t)2 * n * sizeof(pv::QtArgs<double>), kAlign);
         B.off_qtoff = off;
-        off += align_up((size_t)3 * (n + 1) * sizeof(int), kAlign);
+        off += align_up((size_t)2 * (n + 1) * sizeof(int), kAlign);
     }
     B.total = off;
     return B;
@@ -1297,12 +1308,12 @@ pixvod_status batch_launched(pixvod_batch* b) {
 }
 
 // quadtree batches: every sequence's sweep arguments for cur = 0 and cur = 1,
-// and the three kernels' prefix sums of blocks per sequence
+// and the two kernels' prefix sums of blocks per sequence
 template <typename T>
 pixvod_status upload_qt(pixvod_batch* b) {
     const int n = b->n;
     std::vector<pv::QtArgs<T>> args(2 * (size_t)n);
-    std::vector<int> off(3 * (size_t)(n + 1), 0);
+    std::vector<int> off(2 * (size_t)(n + 1), 0);
     for (int i = 0; i < n; ++i) {
         pixvod_handle* h = &b->seq[i];
         const int keep = h->cur;
@@ -1311,12 +1322,10 @@ pixvod_status upload_qt(pixvod_batch* b) {
             args[(size_t)c * n + i] = qt_args<T>(h);
         }
         h->cur = keep;
-        const dim3 pg = pixel_grid(h);
-        off[i + 1] = off[i] + (int)(pg.x * pg.y);
-        off[(n + 1) + i + 1] = off[(n + 1) + i] + (int)qt_msg_blocks(h);
-        off[2 * (n + 1) + i + 1] = off[2 * (n + 1) + i] + (h->L.q.n_nodes + 127) / 128;
+        off[i + 1] = off[i] + qt_message_blocks(h);
+        off[(n + 1) + i + 1] = off[(n + 1) + i] + qt_belief_blocks(h);
     }
-    for (int k = 0; k < 3; ++k) b->qt_blocks[k] = off[k * (n + 1) + n];
+    for (int k = 0; k < 2; ++k) b->qt_blocks[k] = off[k * (n + 1) + n];
     pixvod_status s = cuda_status(cudaMemcpyAsync(b->ws + b->off_qtargs, args.data(), args.size() * sizeof(args[0]),
                                                   cudaMemcpyHostToDevice, b->stream));
     if (s == PIXVOD_OK)
@@ -1326,18 +1335,16 @@ pixvod_status upload_qt(pixvod_batch* b) {
     return s;
 }
 
-// one synchronous sweep of every quadtree sequence: three launches
+// one synchronous sweep of every quadtree sequence: two launches
 template <typename T>
 pixvod_status batch_qt_sweep(pixvod_batch* b, int cur) {
     const pv::QtArgs<T>* A = reinterpret_cast<const pv::QtArgs<T>*>(b->ws + b->off_qtargs) + (size_t)cur * b->n;
     const int* off = reinterpret_cast<const int*>(b->ws + b->off_qtoff);
     const int n = b->n;
-    pv::k_qt_pixels<T><<<b->qt_blocks[0], pixel_block(), 0, b->stream>>>(A, off, n);
+    launch_pdl(pv::k_qt_messages<T>, dim3(b->qt_blocks[0]), pixel_block(), 0, b->stream, A, off, n);
     pixvod_status s = batch_launched(b);
     if (s != PIXVOD_OK) return s;
-    pv::k_qt_node_msgs<T><<<b->qt_blocks[1], 128, 0, b->stream>>>(A, off + (n + 1), n);
-    if ((s = batch_launched(b)) != PIXVOD_OK) return s;
-    pv::k_qt_node_belief<T><<<b->qt_blocks[2], 128, 0, b->stream>>>(A, off + 2 * (n + 1), n);
+    launch_pdl(pv::k_qt_node_belief<T>, dim3(b->qt_blocks[1]), dim3(128), 0, b->stream, A, off + (n + 1), n);
     return batch_launched(b);
 }
 
@@ -1535,7 +1542,7 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
     b->off_qtargs = B.off_qtargs;
     b->off_qtoff = B.off_qtoff;
     b->qt = p->topology == PIXVOD_TOPOLOGY_QUADTREE;
-    b->qt_blocks[0] = b->qt_blocks[1] = b->qt_blocks[2] = 0;
+    b->qt_blocks[0] = b->qt_blocks[1] = 0;
     b->n_work = B.n_work;
     b->schedule = PIXVOD_SCHED_PERSISTENT;
     b->wait_limit = pv::GRID_SYNC_DEFAULT_LIMIT;
@@ -1568,6 +1575,7 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
         h.rec_n = 0;
         h.rec_window = 0;
         h.rec_valid = false;
+        h.qt_stale = false;
     }
     int dev = 0;
     s = cuda_status(cudaGetDevice(&dev));

@@ -619,22 +619,24 @@ PV_HD void sym6_mv(const T* S, const T* x, T* y) {
 // solve was one dependent chain (the sweep waits on its chains, not on a pipe),
 // and a smaller rounding error (random W of up to seven messages with eigenvalues
 // 1e-5..1 lam: 0.8-1.2e-7 normwise in Lambda against 0.9-1.4e-7 before).
-template <typename T>
+// U false: no rank-one part (u = 0, a pose node as the sender; the same values).
+template <typename T, bool U = true>
 struct IdMsg {
     T Ai[21];      // A^-1
     T dg[6];       // (A^-1 W)_rr
     T z[6], zi[6]; // z and z / (1 + u^T z)
     T he[6];       // eta / lam
     // C^-1, entry (r, c); off the diagonal -Lambda / lam^2
-    PV_HD T ci(int r, int c) const { return v_fma(-zi[c], z[r], Ai[pidx(r, c)]); }
+    PV_HD T ci(int r, int c) const { return U ? v_fma(-zi[c], z[r], Ai[pidx(r, c)]) : Ai[pidx(r, c)]; }
     // w Lambda + b, entry (r, c), r >= c, with the products wl = w lam, wll = w lam^2
     PV_HD T lambda(int r, int c, T wl, T wll, T b) const {
-        return r == c ? v_fma(wl, dg[r], v_fma(wll * zi[r], z[r], b)) : v_fma(-wll, ci(r, c), b);
+        if (r != c) return v_fma(-wll, ci(r, c), b);
+        return v_fma(wl, dg[r], U ? v_fma(wll * zi[r], z[r], b) : b);
     }
 };
 
-template <typename T>
-PV_HD bool identity_msg(const T* W, const T* u, const T* etav, const T* r, T lam, IdMsg<T>& m) {
+template <typename T, bool U>
+PV_HD bool identity_msg(const T* W, const T* u, const T* etav, const T* r, T lam, IdMsg<T, U>& m) {
     T A[21], g[6], h[6];
 #pragma unroll
     for (int q = 0; q < 21; ++q) A[q] = W[q];
@@ -653,8 +655,13 @@ PV_HD bool identity_msg(const T* W, const T* u, const T* etav, const T* r, T lam
         }
         m.dg[q] = v_fma(m.Ai[pidx(q, q)], W[pidx(q, q)], s);
     }
-    sym6_mv(m.Ai, u, m.z);
     sym6_mv(m.Ai, g, h);
+    if constexpr (!U) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) m.he[q] = h[q];
+        return ok;
+    }
+    sym6_mv(m.Ai, u, m.z);
     T uz = u[0] * m.z[0], ur = u[0] * r[0], uh = u[0] * h[0];
 #pragma unroll
     for (int q = 1; q < 6; ++q) {

@@ -1,10 +1,12 @@
 // Sweep with the hierarchical (quadtree) identity topology (Sec. 3.3 factor
 // graph; Sec. 4.2: sigma_R and sigma_P halved per level). Pixels keep the state
 // layout of the grid sweep, using identity slot 0 for the factor to their level-1
-// node; pose nodes of every level live in one structure-of-arrays buffer. One
-// synchronous sweep = k_qt_pixels + k_qt_node_msgs + k_qt_node_belief: the first
-// two read only the `in` buffers, the third the node messages the second wrote,
-// and all write the `out` buffers.
+// node (slots 1..3 are zero in both state buffers from the start and are not
+// written: 324 of a pixel's 604 bytes); pose nodes of every level live in one
+// structure-of-arrays buffer. One synchronous sweep = k_qt_messages +
+// k_qt_node_belief: the first (pixel updates and the messages into the nodes)
+// reads only the `in` buffers, the second the node messages the first wrote, and
+// both write the `out` buffers.
 #pragma once
 
 #include "pv_kernels.cuh"
@@ -95,7 +97,6 @@ __device__ __forceinline__ void qt_pixels(const QtArgs<T>& a, int bx, int by) {
         const T* N = a.nin + n;
         const size_t st = q.stride;
         T xs[6], W[21], ev[6], rb[6];
-        const T zero6[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
 #pragma unroll
         for (int c = 0; c < 6; ++c) xs[c] = N[(NP_MU + c) * st];
         const T* mk = N + (NP_MSG + ID_STRIDE * k) * st;
@@ -104,8 +105,8 @@ __device__ __forceinline__ void qt_pixels(const QtArgs<T>& a, int bx, int by) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) ev[c] = -mk[(21 + c) * st];
         se3_between(xs, qi, t, rb);
-        IdMsg<T> m;
-        if (!identity_msg(W, zero6, ev, rb, F.lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
+        IdMsg<T, false> m;
+        if (!identity_msg(W, xs, ev, rb, F.lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
         const T* old = Si + PL_ID * TILE_PX;
         const T wl = omb * F.lam_R, wll = wl * F.lam_R;
 #pragma unroll
@@ -273,8 +274,6 @@ __device__ __forceinline__ void qt_pixels(const QtArgs<T>& a, int bx, int by) {
             for (int c = 0; c < 6; ++c) e -= Lnew[pidx(r, c)] * tau[c];
             d0[(21 + r) * TILE_PX] = e;
         }
-#pragma unroll 1
-        for (int q = ID_STRIDE; q < MSG_PLANES; ++q) d0[q * TILE_PX] = T(0);
     }
     if (flags) atomicOr(&a.sc->flags, flags);
 }
@@ -288,7 +287,7 @@ __device__ __forceinline__ int qt_level(const QtGeom& q, int n) {
 
 // Node update, in two launches per sweep. A node's five messages (children
 // 0..3, parent 4) are independent given the input state, so they are computed by
-// one thread each (k_qt_node_msgs); one thread per node then forms the belief,
+// one thread each (k_qt_messages); one thread per node then forms the belief,
 // updates the pose and projects the messages (k_qt_node_belief). With one thread
 // per node doing all five slots in sequence, the 102k nodes of a 640x480 image
 // fit in a single wave and the sweep waited on that chain of dependent
@@ -327,7 +326,7 @@ __device__ __forceinline__ void qt_node_msgs(const QtArgs<T>& a, int blk) {
     const Geometry<T>& g = a.g;
     const Factors<T>& F = a.f;
     const size_t st = q.stride;
-    const size_t gid = (size_t)blk * blockDim.x + threadIdx.x;
+    const size_t gid = (size_t)blk * TILE_PX + threadIdx.y * TILE_W + threadIdx.x;
     const int tiles_y = (g.H + TILE_H - 1) / TILE_H;
     const size_t n_px = (size_t)g.tiles_x * tiles_y * TILE_PX;
     const int n_up = q.n_levels > 1 ? q.n_nodes - q.base[1] : 0;     // nodes of levels >= 2
@@ -444,7 +443,7 @@ __device__ __forceinline__ void qt_node_msgs(const QtArgs<T>& a, int blk) {
 }
 
 // One thread per node: belief = pose prior (sigma_P / 2^l) plus the five damped
-// messages k_qt_node_msgs left in the output slots (summed in slot order), belief
+// messages k_qt_messages left in the output slots (summed in slot order), belief
 // solve, Exp/Log update, and eta <- eta - Lambda tau on every slot in place.
 template <typename T>
 __device__ __forceinline__ void qt_node_belief(const QtArgs<T>& a, int blk) {
@@ -538,28 +537,29 @@ __device__ __forceinline__ int batch_seq(const int* __restrict__ off, int n, int
     return lo;
 }
 
+// Blocks of k_qt_messages within a sequence: one per 32 x 4 pixels, then the
+// node messages' (independent of the pixels', so one launch holds both).
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 1) k_qt_pixels(const QtArgs<T>* __restrict__ A,
-                                                         const int* __restrict__ off, int n) {
+__global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? 4 : 2) k_qt_messages(const QtArgs<T>* __restrict__ A,
+                                                                                 const int* __restrict__ off, int n) {
     const int i = batch_seq(off, n, blockIdx.x);
     const QtArgs<T>& a = A[i];
-    const int lb = blockIdx.x - __ldg(off + i);
-    const int gx = (a.g.W + (int)blockDim.x - 1) / (int)blockDim.x;
-    qt_pixels(a, lb % gx, lb / gx);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(128, 4) k_qt_node_msgs(const QtArgs<T>* __restrict__ A,
-                                                               const int* __restrict__ off, int n) {
-    const int i = batch_seq(off, n, blockIdx.x);
-    qt_node_msgs(A[i], blockIdx.x - __ldg(off + i));
+    const int lb = blockIdx.x - __ldg(off + i), px = a.g.tiles_x * ((a.g.H + TILE_H - 1) / TILE_H);
+    pdl_wait();
+    if (lb < px)
+        qt_pixels(a, lb % a.g.tiles_x, lb / a.g.tiles_x);
+    else
+        qt_node_msgs(a, lb - px);
+    pdl_trigger();
 }
 
 template <typename T>
 __global__ void __launch_bounds__(128) k_qt_node_belief(const QtArgs<T>* __restrict__ A,
                                                               const int* __restrict__ off, int n) {
     const int i = batch_seq(off, n, blockIdx.x);
+    pdl_wait();
     qt_node_belief(A[i], blockIdx.x - __ldg(off + i));
+    pdl_trigger();
 }
 
 // Keyframe reset of every node: identity pose, belief = the level's pose prior,
