@@ -15,10 +15,12 @@
 #include "../../include/pixvod.h"
 #include "pv_adjoint_api.h"
 #include "pv_batch.cuh"
+#include "pv_launch.h"
 #include "pv_quadtree.cuh"
 
 using pv::Factors;
 using pv::Geometry;
+using pv::launch_pdl;
 using pv::Scalars;
 
 namespace {
@@ -308,23 +310,6 @@ cudaError_t sweep_attributes() {
     static cudaError_t once = cudaFuncSetAttribute(pv::k_sweeps<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)pv::sweep_smem_bytes<T>());
     return once;
-}
-
-// launch on `st` with programmatic stream serialization: the kernel may be
-// scheduled while its predecessor drains (it waits for it itself, pv::pdl_wait)
-template <typename... P, typename... A>
-void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // the error is read by cudaGetLastError
 }
 
 // one synchronous grid sweep: the tiles of `work` (null: of the descriptor's
@@ -628,7 +613,7 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
     double* dparam = misc;                                                        // 3 doubles
     unsigned long long* mism = reinterpret_cast<unsigned long long*>(misc + 4);  // 1
     unsigned* fl = reinterpret_cast<unsigned*>(misc + 5);                        // flags, max nodes
-    double* scale = misc + 8;  // exponent of the adjoint state's units, max |adjoint| (2 doubles)
+    double* scale = misc + 8;  // exponent of the adjoint state's units and the pass's factors (6 doubles)
     pixvod_status s = cuda_status(sweep_attributes<T>());
     if (s == PIXVOD_OK) s = cuda_status(cudaMemsetAsync(dIs, 0, npx * sizeof(double), st));
     if (s == PIXVOD_OK) s = cuda_status(cudaMemsetAsync(dIt, 0, npx * sizeof(double), st));
@@ -716,15 +701,13 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
             if ((r = cuda_status(pv::launch_adjoint_sweep(A, R.slots / pv::ad::ADJ_THREADS, st))) != PIXVOD_OK)
                 return r;
         } else {
-            // rescale by a power of two: max |adj_out| (which also zeroes adj_in;
-            // scale[1] is 0 from the start of the backward or the last exponent),
-            // the pass, the new exponent
-            h->launches += 2 + pv::ADJOINT_HW_LAUNCHES;  // absmax, the pass, the exponent
+            // rescale by a power of two: max |adj_out| and the factors (which also
+            // zeroes adj_in), then the pass
+            h->launches += 1 + pv::ADJOINT_HW_LAUNCHES;
             if ((r = cuda_status(pv::launch_adjoint_absmax(adj[a], adj[a ^ 1], adj_elems, adj64 ? 1 : 0, scale,
                                                            st))) != PIXVOD_OK)
                 return r;
             if ((r = cuda_status(pv::launch_adjoint_hw(A, n_tiles, rw + R.off_scr, st))) != PIXVOD_OK) return r;
-            if ((r = cuda_status(pv::launch_adjoint_exponent(scale, st))) != PIXVOD_OK) return r;
         }
         a ^= 1;
         return PIXVOD_OK;

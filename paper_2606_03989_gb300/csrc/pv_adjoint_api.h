@@ -49,10 +49,10 @@ struct AdjArgs {
     unsigned* max_nodes;           // longest tape of a pixel
     unsigned* flags;
     ad::TapeCtl tape;
-    // hand-written pass: scale[0] = E, the adjoint state holds values in units
-    // of 2^E; scale[1] = max |adj_out| in those units (as written by
-    // launch_adjoint_absmax); the pass reads adj_out times 2^-e with
-    // e = ilogb(scale[1]), so its adj_in is in units of 2^(E + e)
+    // hand-written pass (scale[0..5], zero before the first): the adjoint state
+    // holds values in units of 2^E, E = scale[0]; the pass reads adj_out times
+    // scale[2] = 2^-e with e = ilogb(max |adj_out|), so its adj_in is in units of
+    // scale[3] = 2^(E + e) (launch_adjoint_absmax sets both and adds e to E)
     double* scale;
 };
 
@@ -61,12 +61,12 @@ struct AdjArgs {
 cudaError_t launch_adjoint_sweep(const AdjArgs& A, int blocks, cudaStream_t st);
 // adjoint of one sweep by the hand-written reverse pass, in the state's
 // precision, as ADJOINT_HW_LAUNCHES launches: per pixel and direction (the
-// damped identity messages and what their reverse needs, summed over the
-// directions), per pixel (the update and the reverse pass of everything but the
-// identity messages), per pixel and direction (the identity messages' reverse
-// pass), per tile (the recompute check), per pixel (the pose); `scratch`
-// (adjoint_scratch_bytes) carries values between them
-constexpr int ADJOINT_HW_LAUNCHES = 5;
+// damped identity messages summed over the directions), per pixel (the update and
+// the reverse pass of everything but the identity messages), per pixel and
+// direction (the identity messages' reverse pass), per pixel (the pose), each with
+// its part of the recompute check; `scratch` (adjoint_scratch_bytes) carries values
+// between them
+constexpr int ADJOINT_HW_LAUNCHES = 4;
 size_t adjoint_scratch_bytes(int n_tiles, int state64);
 cudaError_t launch_adjoint_hw(const AdjArgs& A, int n_tiles, void* scratch, cudaStream_t st);
 // adjoint of xi_est = mean mu[0:6] and of the inverse depth exp(-mu[6]) at the
@@ -74,12 +74,9 @@ cudaError_t launch_adjoint_hw(const AdjArgs& A, int n_tiles, void* scratch, cuda
 // (adj64) or FP32
 cudaError_t launch_adjoint_seed(const AdjArgs& A, const double* grad_xi, const double* grad_invdepth, void* adj,
                                 int adj64, cudaStream_t st);
-// scale[1] = max |a[i]| over n elements (finite values; scale[1] must be 0 before),
-// and z[i] = 0 over the same n elements (the next pass's adj_in)
+// the scale factors of the pass that reads a (AdjArgs::scale), from max |a[i]| over
+// n elements (finite values), and z[i] = 0 over the same n elements (its adj_in)
 cudaError_t launch_adjoint_absmax(const void* a, void* z, size_t n, int adj64, double* scale, cudaStream_t st);
-// scale[0] += ilogb(scale[1]): the units of the adjoint state after a hand-written
-// pass; scale[1] = 0 again for the next pass's absmax
-cudaError_t launch_adjoint_exponent(double* scale, cudaStream_t st);
 // dL/d(sigma_D, sigma_N) from the adjoints of lam_D, 1/sigma_D and lam_N
 cudaError_t launch_sigma_grads(const double* dparam, double sigma_D, double sigma_N, double* out, cudaStream_t st);
 
