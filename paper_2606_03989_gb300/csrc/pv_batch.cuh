@@ -24,7 +24,16 @@ struct SeqDesc {
     const float* normals;
     unsigned char* br;     // decisions of the sweep, recorded for the adjoint (or null)
     int n_tiles;
+    int rows;              // the sweep's work items are rows of tiles (4 tile + row), not tiles
 };
+
+// An image of at most this many tiles is swept by rows (sweep_row): two tiles per
+// SM in FP32 (measured: faster at 280 tiles, slower at 384), half a tile in FP64
+// (the rows then fit on the SMs at once; faster at 24 and 48 tiles, slower at 96).
+template <typename T>
+constexpr int row_mode_tiles() {
+    return sizeof(T) == 4 ? 304 : 76;
+}
 
 struct Work {
     int seq;
@@ -46,6 +55,7 @@ __device__ __forceinline__ SweepArgs<T> seq_args(const SeqDesc<T>& d, int cur) {
     a.m_y = d.in_planes[5];
     a.sc = d.sc;
     a.br = d.br;
+    a.rows = d.rows;
     return a;
 }
 
@@ -90,7 +100,7 @@ __device__ __forceinline__ bool grid_sync(const GridSync& gs) {
     return ok_sh != 0;
 }
 
-// Synchronous sweeps over a list of (sequence, tile) work items. This one kernel
+// Synchronous sweeps over a list of (sequence, tile or row of a tile) work items. This one kernel
 // serves every schedule, so a tile's arithmetic is the same machine code however
 // the work is launched (and the results do not depend on the schedule):
 //  - one sweep per launch, one block per work item (n_iters == 1, grid == n_work);
@@ -124,12 +134,16 @@ __global__ void __launch_bounds__(SWEEP_THREADS, sizeof(T) == 4 ? 4 : 2) k_sweep
             const int w = flip ? n_work - 1 - k : k;
             const Work wk = work ? work[w] : Work{0, w};
             const SweepArgs<T> a = seq_args(seqs[wk.seq], cur);
+            const int tile = a.rows ? wk.tile / TILE_H : wk.tile, tx = tile % a.g.tiles_x, ty = tile / a.g.tiles_x;
+            if (a.rows) {
+                sweep_row(a, tx, ty, wk.tile % TILE_H, msg, it + 1 == n_iters);
+                __syncthreads();
+                continue;
+            }
             // a tile whose bulk copy never arrived ends the block's work for the
             // launch: the mbarrier's phase no longer matches `parity`, and the copy
             // may still be writing `msg`
-            if (!sweep_tile(a, wk.tile % a.g.tiles_x, wk.tile / a.g.tiles_x, msg, &bar, parity,
-                            it + 1 == n_iters))
-                return;
+            if (!sweep_tile(a, tx, ty, msg, &bar, parity, it + 1 == n_iters)) return;
             parity ^= 1u;
             if (n_iters > 1) asm volatile("fence.proxy.async.global;" ::: "memory");
             __syncthreads();

@@ -110,6 +110,7 @@ struct SweepArgs {
     // when set, each pixel's discrete decisions of this sweep (BR_* bits) are
     // written here (tile-major pixel index), for the adjoint
     unsigned char* br;
+    int rows;  // work items are rows of tiles (sweep_row), not tiles
 };
 
 
@@ -309,57 +310,21 @@ constexpr size_t sweep_smem_bytes() {
     return sizeof(T) * LAM_PLANES * TILE_PX;
 }
 
-// The calling thread's pixel of the sweep over tile (tx, ty): everything but the
-// store of the identity messages' Lambda, which are left in `msg`. False if the
-// tile's bulk copy never arrived (FLAG_TIMEOUT is set).
+// a1: photometric factor (Eqs. 2, 3) of pixel (u, v), input-plane index i, at the
+// mean (qi, t, d)
 template <typename T>
-__device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int ty, T* msg, uint64_t* bar,
-                                            unsigned parity) {
-    const int tid = threadIdx.y * SWEEP_BX + threadIdx.x;
-    const int u = tx * SWEEP_BX + threadIdx.x;
-    const int v = ty * SWEEP_BY + threadIdx.y;
+__device__ __forceinline__ void photometric_factor(const SweepArgs<T>& a, int i, int u, int v, const T* qi, const T* t,
+                                                   T d, T* J, T& alpha, T& rph, unsigned char& br, unsigned& flags) {
     const Geometry<T>& g = a.g;
     const Factors<T>& F = a.f;
-    const size_t tile = (size_t)ty * g.tiles_x + tx;
-    if (u >= g.W || v >= g.H) return true;
-    unsigned flags = 0;
-    const size_t n_state = (size_t)g.tiles_x * ((g.H + TILE_H - 1) / TILE_H) * TILE_WORDS;
     const size_t n_plane = g.plane;
-    (void)n_state;
     (void)n_plane;
-    const int i = (int)PV_IDX(v * g.pitch + u, n_plane, flags);
-    const T* __restrict__ Si = a.in + PV_IDX(tile * TILE_WORDS + tid, n_state, flags);   // this pixel, plane 0
-    T* __restrict__ Di = a.out + PV_IDX(tile * TILE_WORDS + tid, n_state, flags);
-
-    T xi[6], d;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) xi[k] = ld_state(Si + k * TILE_PX);
-    d = ld_state(Si + 6 * TILE_PX);
-    T qi[4], t[3];
-    se3_exp_q(xi, qi, t);
-
-    // The belief has the exact structure
-    //   Lambda_b = blockdiag(M_p, m_d) + alpha J J^T,  eta_b = eta_o - alpha r J
-    // (identity messages and the pose prior act on the pose block, normal messages
-    // and the depth prior on the depth, the photometric factor is rank one), so it
-    // is kept in that form: M_p (packed), m_d, alpha, J, r and eta_o (in eb).
-    T eb[7];
-#pragma unroll
-    for (int q = 0; q < 7; ++q) eb[q] = T(0);
-    // --- priors (Eq. 4 with identity Jacobian; log-depth prior) ---
-#pragma unroll
-    for (int k = 0; k < 6; ++k) eb[k] -= F.lam_P * xi[k];
-    T md = F.lam_Z;
-    eb[6] -= F.lam_Z * (d - T(a.sc->d_prior));
-
-    T alpha = T(0), rph = T(0);
-    T J[7];
+    (void)flags;
+    alpha = T(0);
+    rph = T(0);
+    br = 0;
 #pragma unroll
     for (int q = 0; q < 7; ++q) J[q] = T(0);
-    unsigned char br = 0;
-
-    // --- a1: photometric factor (Eqs. 2, 3) at the current mean (it enters only
-    // the belief below, so it is evaluated after the pairwise messages) ---
     {
         T R[9];
         quat_matrix(qi, R);
@@ -421,115 +386,80 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
             br = hub ? (BR_VALID | BR_HUBER) : BR_VALID;
         }
     }
-    // --- a2/a3: pairwise messages from the four neighbours ---
-    if (!mbar_wait_bounded(bar, parity)) {
-        // the tile's messages never arrived: flag it, wait once more, leave the tile
-        atomicOr(&a.sc->flags, FLAG_TIMEOUT);
-        mbar_wait_bounded(bar, parity);
-        return false;
+}
+
+// The neighbour of (u, v) in direction k (left, right, up, down)
+template <typename T>
+__device__ __forceinline__ bool sweep_neighbour(const Geometry<T>& g, int u, int v, int k, int* un, int* vn) {
+    *un = u + (k == 0 ? -1 : (k == 1 ? 1 : 0));
+    *vn = v + (k == 2 ? -1 : (k == 3 ? 1 : 0));
+    return *un >= 0 && *un < g.W && *vn >= 0 && *vn < g.H;
+}
+
+// a2/a3: the identity message from the neighbour in direction k, its state at Sj.
+// Its variable-to-factor marginal is V = W + u u^T with W = M_p,j - Lambda_{f->j}
+// (pose prior plus j's three other identity messages), u = u_j and eta_v =
+// -eta_{f->j}. All loads (also the old eta of the pixel's message, eo) are issued
+// ahead of the Exp/Log chain of the residual, so that their latency overlaps it.
+template <typename T>
+__device__ __forceinline__ void sweep_message(const T* Si, const T* Sj, int k, const T* qi, const T* t, T lam_R,
+                                              IdMsg<T>& m, T* eo, unsigned& flags) {
+    const T* mj = Sj + (PL_ID + ID_STRIDE * (k ^ 1)) * TILE_PX;
+    T W[21], uj[6], gv[6], xj[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) xj[q] = ld_state(Sj + q * TILE_PX);
+#pragma unroll
+    for (int q = 0; q < 21; ++q) W[q] = ld_state(Sj + (PL_MP + q) * TILE_PX) - ld_state(mj + q * TILE_PX);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        uj[q] = ld_state(Sj + (PL_U + q) * TILE_PX);
+        gv[q] = -ld_state(mj + (LAM + q) * TILE_PX);
     }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) eo[q] = ld_state(Si + (PL_ID + ID_STRIDE * k + LAM + q) * TILE_PX);
+    T rb[6];
+    se3_between(xj, qi, t, rb);
+    if (!identity_msg(W, uj, gv, rb, lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
+}
+
+// a3': the normal-integration message (Eq. 6: r_i = d_i - d_j + sg m) from the
+// neighbour in direction k, its state at Sj
+template <typename T>
+__device__ __forceinline__ void sweep_normal(const SweepArgs<T>& a, const T* Si, const T* Sj, int k, int i, T d, T* nl,
+                                             T* ne, unsigned& flags) {
+    const Geometry<T>& g = a.g;
+    const Factors<T>& F = a.f;
     const T beta = F.beta, omb = T(1) - F.beta;
-#pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
-        T* mb = msg + PV_IDX((k * LAM) * TILE_PX + tid, (LAM_PLANES - LAM + 1) * TILE_PX, flags);  // slot k
-        T* me = Di + (PL_ID + ID_STRIDE * k + LAM) * TILE_PX;                                                    // its eta
-        const int un = u + (k == 0 ? -1 : (k == 1 ? 1 : 0));
-        const int vn = v + (k == 2 ? -1 : (k == 3 ? 1 : 0));
-        const bool has = un >= 0 && un < g.W && vn >= 0 && vn < g.H;
-        if (!has) {
-#pragma unroll
-            for (int q = 0; q < 21; ++q) mb[q * TILE_PX] = T(0);
-#pragma unroll
-            for (int q = 0; q < 6; ++q) me[q * TILE_PX] = T(0);
-            continue;
-        }
-        const int ko = k ^ 1;
-        const T* Sj = a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags);
-        // variable-to-factor marginal of j: V = W + u u^T with W = M_p,j - Lambda_{f->j}
-        // (pose prior plus j's three other identity messages) and u = u_j, and
-        // eta_v = -eta_{f->j}. All of j's loads are issued here, ahead of the Exp/Log
-        // chain of the residual, so that their latency overlaps it.
-        const T* mj = Sj + (PL_ID + ID_STRIDE * ko) * TILE_PX;
-        T W[21], uj[6], gv[6], xj[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) xj[q] = ld_state(Sj + q * TILE_PX);
-#pragma unroll
-        for (int q = 0; q < 21; ++q) W[q] = ld_state(Sj + (PL_MP + q) * TILE_PX) - ld_state(mj + q * TILE_PX);
-#pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            uj[q] = ld_state(Sj + (PL_U + q) * TILE_PX);
-            gv[q] = -ld_state(mj + (21 + q) * TILE_PX);
-        }
-        T eo[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) eo[q] = ld_state(Si + (PL_ID + ID_STRIDE * k + LAM + q) * TILE_PX);
-        T rb[6];
-        se3_between(xj, qi, t, rb);
-        IdMsg<T> m;
-        if (!identity_msg(W, uj, gv, rb, F.lam_R, m)) flags |= FLAG_NONPOS_PIVOT;
-        // damped: (1 - beta) new + beta old; Lambda over the old one in shared memory
-        const T wl = omb * F.lam_R, wll = wl * F.lam_R;
-#pragma unroll
-        for (int q = 0; q < 6; ++q) {
-            const T e = v_fma(wl, m.he[q], beta * eo[q]);
-            eb[q] += e;
-            me[q * TILE_PX] = e;
-        }
-#pragma unroll
-        for (int c = 0; c < 6; ++c)
-#pragma unroll
-            for (int r = c; r < 6; ++r) {
-                const T l = m.lambda(r, c, wl, wll, beta * mb[pidx(r, c) * TILE_PX]);
-                mb[pidx(r, c) * TILE_PX] = l;
-            }
-    }
-    // M_p from the four messages in shared memory
-    T Mp[21];
-#pragma unroll
-    for (int q = 0; q < 21; ++q) {
-        T x = T(0);
-#pragma unroll
-        for (int k = 0; k < 6; ++k)
-            if (q == pidx(k, k)) x = F.lam_P;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) x += msg[(LAM * k + q) * TILE_PX + tid];
-        Mp[q] = x;
-    }
+    const size_t n_plane = g.plane;
+    (void)n_plane;
+    (void)flags;
+    const int ko = k ^ 1;
+    T dj = ld_state(Sj + 6 * TILE_PX);
+    T sv = ld_state(Sj + PL_S * TILE_PX) - ld_state(Sj + (PL_NM + 2 * ko) * TILE_PX);
+    T evn = -ld_state(Sj + (PL_NM + 2 * ko + 1) * TILE_PX);
+    T m = k == 0 ? a.m_x[PV_IDX(i - 1, n_plane, flags)]
+                 : (k == 1 ? a.m_x[i] : (k == 2 ? a.m_y[PV_IDX(i - g.pitch, n_plane, flags)] : a.m_y[i]));
+    T sg = (k == 0 || k == 2) ? T(1) : T(-1);
+    T rn = d - dj + sg * m;
+    T den = v_div(T(1), F.lam_N + sv);
+    *nl = omb * (F.lam_N * sv * den) + beta * ld_state(Si + (PL_NM + 2 * k) * TILE_PX);
+    *ne = omb * (F.lam_N * (evn - sv * rn) * den) + beta * ld_state(Si + (PL_NM + 2 * k + 1) * TILE_PX);
+}
 
-    // normal-integration factors (Eq. 6): r_i = d_i - d_j + sg m
-    T nl[4], ne[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        nl[k] = T(0);
-        ne[k] = T(0);
-        const int un = u + (k == 0 ? -1 : (k == 1 ? 1 : 0));
-        const int vn = v + (k == 2 ? -1 : (k == 3 ? 1 : 0));
-        if (!(un >= 0 && un < g.W && vn >= 0 && vn < g.H)) continue;
-        const int ko = k ^ 1;
-        const T* Sj = a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags);
-        T dj = ld_state(Sj + 6 * TILE_PX);
-        T sv = ld_state(Sj + PL_S * TILE_PX) - ld_state(Sj + (PL_NM + 2 * ko) * TILE_PX);
-        T evn = -ld_state(Sj + (PL_NM + 2 * ko + 1) * TILE_PX);
-        T m = k == 0 ? a.m_x[PV_IDX(i - 1, n_plane, flags)]
-                     : (k == 1 ? a.m_x[i] : (k == 2 ? a.m_y[PV_IDX(i - g.pitch, n_plane, flags)] : a.m_y[i]));
-        T sg = (k == 0 || k == 2) ? T(1) : T(-1);
-        T rn = d - dj + sg * m;
-        T den = v_div(T(1), F.lam_N + sv);
-        nl[k] = omb * (F.lam_N * sv * den) + beta * ld_state(Si + (PL_NM + 2 * k) * TILE_PX);
-        ne[k] = omb * (F.lam_N * (evn - sv * rn) * den) + beta * ld_state(Si + (PL_NM + 2 * k + 1) * TILE_PX);
-        md += nl[k];
-        eb[6] += ne[k];
-    }
-
-    // --- a4: belief, mean update, tangent projection ---
+// a4: the mean update tau from the belief
+//   Lambda_b = blockdiag(M_p, m_d) + alpha J J^T,  eta_b = eta_o - alpha r J
+// (identity messages and the pose prior act on the pose block, normal messages
+// and the depth prior on the depth, the photometric factor is rank one), which is
+// kept in that form: M_p (packed), m_d, alpha, J, r and eta_o (in eb). qv: q below.
+template <typename T>
+__device__ __forceinline__ void belief_update(const T* Mp, T md, const T* eb, const T* J, T alpha, T rph, T* tau, T& qv,
+                                              unsigned char& br, unsigned& flags) {
     // With B = blockdiag(M_p, m_d), h = B^-1 eta_o and z = B^-1 J, Sherman-Morrison
     // gives tau = Lambda_b^-1 eta_b = h - z alpha (r + J^T h) / (1 + alpha J^T z),
     // and the marginals of Lambda_b are, with q = J_p^T M_p^-1 J_p,
     //   P = M_p + u u^T,  u = sqrt(alpha m_d / (m_d + alpha J_d^2)) J_p,
     //   s = m_d + alpha J_d^2 / (1 + alpha q),
     // all free of cancellation.
-    T tau[7];
-    T qv;
     bool ok;
     {
         T Lp[21], idp[6];
@@ -571,6 +501,117 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
 #pragma unroll
         for (int q = 0; q < 7; ++q) tau[q] = T(0);
     }
+}
+
+// The belief's marginals besides M_p: u = sb J_p (the photometric part of the
+// depth-marginalised pose information) and s (pose-marginalised depth information)
+template <typename T>
+__device__ __forceinline__ void depth_marginals(T md, T alpha, T Jd, T qv, T* sb, T* s) {
+    const T bp = v_div(alpha * md, md + alpha * Jd * Jd);
+    *sb = v_sqrt(bp);
+    *s = md + v_div(alpha * Jd * Jd, T(1) + alpha * qv);
+}
+
+// The calling thread's pixel of the sweep over tile (tx, ty): everything but the
+// store of the identity messages' Lambda, which are left in `msg`. False if the
+// tile's bulk copy never arrived (FLAG_TIMEOUT is set).
+template <typename T>
+__device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int ty, T* msg, uint64_t* bar,
+                                            unsigned parity) {
+    const int tid = threadIdx.y * SWEEP_BX + threadIdx.x;
+    const int u = tx * SWEEP_BX + threadIdx.x;
+    const int v = ty * SWEEP_BY + threadIdx.y;
+    const Geometry<T>& g = a.g;
+    const Factors<T>& F = a.f;
+    const size_t tile = (size_t)ty * g.tiles_x + tx;
+    if (u >= g.W || v >= g.H) return true;
+    unsigned flags = 0;
+    const size_t n_state = (size_t)g.tiles_x * ((g.H + TILE_H - 1) / TILE_H) * TILE_WORDS;
+    (void)n_state;
+    const int i = (int)PV_IDX(v * g.pitch + u, g.plane, flags);
+    const T* __restrict__ Si = a.in + PV_IDX(tile * TILE_WORDS + tid, n_state, flags);   // this pixel, plane 0
+    T* __restrict__ Di = a.out + PV_IDX(tile * TILE_WORDS + tid, n_state, flags);
+
+    T xi[6], d;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) xi[k] = ld_state(Si + k * TILE_PX);
+    d = ld_state(Si + 6 * TILE_PX);
+    T qi[4], t[3];
+    se3_exp_q(xi, qi, t);
+    // --- priors (Eq. 4 with identity Jacobian; log-depth prior) ---
+    T eb[7];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) eb[k] = -(F.lam_P * xi[k]);
+    T md = F.lam_Z;
+    eb[6] = -(F.lam_Z * (d - T(a.sc->d_prior)));
+
+    T alpha, rph, J[7];
+    unsigned char br;
+    photometric_factor(a, i, u, v, qi, t, d, J, alpha, rph, br, flags);
+
+    if (!mbar_wait_bounded(bar, parity)) {
+        // the tile's messages never arrived: flag it, wait once more, leave the tile
+        atomicOr(&a.sc->flags, FLAG_TIMEOUT);
+        mbar_wait_bounded(bar, parity);
+        return false;
+    }
+    const T beta = F.beta, omb = T(1) - F.beta;
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        T* mb = msg + PV_IDX((k * LAM) * TILE_PX + tid, (LAM_PLANES - LAM + 1) * TILE_PX, flags);  // slot k's Lambda
+        T* me = Di + (PL_ID + ID_STRIDE * k + LAM) * TILE_PX;                                      // its eta
+        int un, vn;
+        if (!sweep_neighbour(g, u, v, k, &un, &vn)) {
+#pragma unroll
+            for (int q = 0; q < LAM; ++q) mb[q * TILE_PX] = T(0);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) me[q * TILE_PX] = T(0);
+            continue;
+        }
+        T eo[6];
+        IdMsg<T> m;
+        sweep_message(Si, a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags), k, qi, t, F.lam_R, m, eo,
+                      flags);
+        // damped: (1 - beta) new + beta old; Lambda over the old one in shared memory
+        const T wl = omb * F.lam_R, wll = wl * F.lam_R;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const T e = v_fma(wl, m.he[q], beta * eo[q]);
+            eb[q] += e;
+            me[q * TILE_PX] = e;
+        }
+#pragma unroll
+        for (int c = 0; c < 6; ++c)
+#pragma unroll
+            for (int r = c; r < 6; ++r)
+                mb[pidx(r, c) * TILE_PX] = m.lambda(r, c, wl, wll, beta * mb[pidx(r, c) * TILE_PX]);
+    }
+    // M_p from the four messages in shared memory
+    T Mp[21];
+#pragma unroll
+    for (int q = 0; q < 21; ++q) {
+        T x = T(0);
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+            if (q == pidx(k, k)) x = F.lam_P;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x += msg[(LAM * k + q) * TILE_PX + tid];
+        Mp[q] = x;
+    }
+    T nl[4], ne[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        nl[k] = T(0);
+        ne[k] = T(0);
+        int un, vn;
+        if (!sweep_neighbour(g, u, v, k, &un, &vn)) continue;
+        sweep_normal(a, Si, a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags), k, i, d, &nl[k], &ne[k],
+                     flags);
+        md += nl[k];
+        eb[6] += ne[k];
+    }
+    T tau[7], qv;
+    belief_update(Mp, md, eb, J, alpha, rph, tau, qv, br, flags);
     if (a.br) a.br[tile * TILE_PX + tid] = br;
     // the new eta, back for the projection below
     T en[24];
@@ -587,13 +628,13 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
         Di[6 * TILE_PX] = d + tau[6];
     }
     {
-        const T bp = v_div(alpha * md, md + alpha * J[6] * J[6]);
-        const T sb = v_sqrt(bp);
+        T sb, s;
+        depth_marginals(md, alpha, J[6], qv, &sb, &s);
 #pragma unroll
         for (int q = 0; q < 21; ++q) Di[(PL_MP + q) * TILE_PX] = Mp[q];
 #pragma unroll
         for (int q = 0; q < 6; ++q) Di[(PL_U + q) * TILE_PX] = sb * J[q];
-        Di[PL_S * TILE_PX] = md + v_div(alpha * J[6] * J[6], T(1) + alpha * qv);
+        Di[PL_S * TILE_PX] = s;
     }
     // messages, projected: eta <- eta - Lambda tau
 #pragma unroll
@@ -614,6 +655,143 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
     }
     if (flags) atomicOr(&a.sc->flags, flags);
     return true;
+}
+
+// The same sweep over row `row` of tile (tx, ty), for images of few tiles: the
+// block's warp k computes the messages of direction k for the row's 32 pixels, the
+// four are summed through shared memory in the same order, and every warp stores
+// its direction's messages and its share of the rest. A tile's latency is one
+// direction's instead of four in turn, on four times as many SMs; that every warp
+// solves the belief costs nothing while the schedulers are idle. Per sweep, by
+// tiles and by rows: 64x48 10.8 and 5.7 us, 128x96 11.4 and 7.7, 160x120 12.6 and
+// 8.2, 224x160 15.0 and 14.1, 256x192 17.2 and 19.6; FP64, bound by its pipe: 64x48
+// 123 and 49, 128x96 123 and 155. Every thread of the block must call it; the caller synchronises
+// the block before `msg` is reused.
+constexpr int ROW_VALUES = 29;  // a direction's Lambda, eta and normal message in shared memory
+template <typename T>
+__device__ __forceinline__ void sweep_row(const SweepArgs<T>& a, int tx, int ty, int row, T* msg, bool last_sweep) {
+    const int k = threadIdx.y, x = threadIdx.x;
+    const int u = tx * TILE_W + x, v = ty * TILE_H + row;
+    const Geometry<T>& g = a.g;
+    const Factors<T>& F = a.f;
+    if (v >= g.H) return;  // the whole block
+    const size_t tile = (size_t)ty * g.tiles_x + tx;
+    const bool inside = u < g.W;
+    unsigned flags = 0;
+    const size_t n_state = (size_t)g.tiles_x * ((g.H + TILE_H - 1) / TILE_H) * TILE_WORDS;
+    (void)n_state;
+    const int lane = row * TILE_W + x;
+    const int i = inside ? (int)PV_IDX(v * g.pitch + u, g.plane, flags) : 0;
+    const T* __restrict__ Si = a.in + PV_IDX(tile * TILE_WORDS + lane, n_state, flags);
+    T* __restrict__ Di = a.out + PV_IDX(tile * TILE_WORDS + lane, n_state, flags);
+    T* sh = msg + k * ROW_VALUES * TILE_W + x;  // this direction's values
+    T xi[6], d = T(0), qi[4], t[3];
+    T alpha = T(0), rph = T(0), J[7];
+    unsigned char br = 0;
+    if (inside) {
+        T l[LAM], e[6], nl = T(0), ne = T(0);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) xi[q] = ld_state(Si + q * TILE_PX);
+        d = ld_state(Si + 6 * TILE_PX);
+#pragma unroll
+        for (int q = 0; q < LAM; ++q) l[q] = ld_state(Si + (PL_ID + ID_STRIDE * k + q) * TILE_PX);  // the old Lambda
+        se3_exp_q(xi, qi, t);
+        int un, vn;
+        if (sweep_neighbour(g, u, v, k, &un, &vn)) {
+            const T beta = F.beta, omb = T(1) - F.beta;
+            const T* Sj = a.in + PV_IDX(state_index(un, vn, g.tiles_x), n_state, flags);
+            sweep_normal(a, Si, Sj, k, i, d, &nl, &ne, flags);
+            T eo[6];
+            IdMsg<T> m;
+            sweep_message(Si, Sj, k, qi, t, F.lam_R, m, eo, flags);
+            const T wl = omb * F.lam_R, wll = wl * F.lam_R;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) e[q] = v_fma(wl, m.he[q], beta * eo[q]);
+#pragma unroll
+            for (int c = 0; c < 6; ++c)
+#pragma unroll
+                for (int r = c; r < 6; ++r) l[pidx(r, c)] = m.lambda(r, c, wl, wll, beta * l[pidx(r, c)]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < LAM; ++q) l[q] = T(0);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) e[q] = T(0);
+        }
+#pragma unroll
+        for (int q = 0; q < LAM; ++q) sh[q * TILE_W] = l[q];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) sh[(LAM + q) * TILE_W] = e[q];
+        sh[27 * TILE_W] = nl;
+        sh[28 * TILE_W] = ne;
+        photometric_factor(a, i, u, v, qi, t, d, J, alpha, rph, br, flags);
+    }
+    __syncthreads();
+    if (last_sweep) pdl_trigger();
+    if (!inside) return;
+    const unsigned mflags = flags;  // this direction's
+    T Mp[21], eb[7], md = F.lam_Z;
+#pragma unroll
+    for (int q = 0; q < 21; ++q) {
+        T y = T(0);
+#pragma unroll
+        for (int j = 0; j < 6; ++j)
+            if (q == pidx(j, j)) y = F.lam_P;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) y += msg[(j * ROW_VALUES + q) * TILE_W + x];
+        Mp[q] = y;
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) eb[q] = -(F.lam_P * xi[q]);
+    eb[6] = -(F.lam_Z * (d - T(a.sc->d_prior)));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const T* sj = msg + j * ROW_VALUES * TILE_W + x;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) eb[q] += sj[(LAM + q) * TILE_W];
+        md += sj[27 * TILE_W];
+        eb[6] += sj[28 * TILE_W];
+    }
+    T tau[7], qv;
+    belief_update(Mp, md, eb, J, alpha, rph, tau, qv, br, flags);
+    T* Dk = Di + (PL_ID + ID_STRIDE * k) * TILE_PX;
+    {
+        T l[LAM];
+#pragma unroll
+        for (int q = 0; q < LAM; ++q) {
+            l[q] = sh[q * TILE_W];
+            Dk[q * TILE_PX] = l[q];
+        }
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+            T y = sh[(LAM + r) * TILE_W];
+#pragma unroll
+            for (int c = 0; c < 6; ++c) y -= l[pidx(r, c)] * tau[c];
+            Dk[(LAM + r) * TILE_PX] = y;
+        }
+        const T nl = sh[27 * TILE_W];
+        Di[(PL_NM + 2 * k) * TILE_PX] = nl;
+        Di[(PL_NM + 2 * k + 1) * TILE_PX] = sh[28 * TILE_W] - nl * tau[6];
+    }
+    if (k == 0) {
+        T xn[6];
+        se3_update(qi, t, tau, xn);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) Di[q * TILE_PX] = xn[q];
+        Di[6 * TILE_PX] = d + tau[6];
+        if (a.br) a.br[tile * TILE_PX + lane] = br;
+    } else if (k == 1) {
+        T sb, s;
+        depth_marginals(md, alpha, J[6], qv, &sb, &s);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) Di[(PL_U + q) * TILE_PX] = sb * J[q];
+        Di[PL_S * TILE_PX] = s;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 21; ++q)
+            if ((q < 10) == (k == 2)) Di[(PL_MP + q) * TILE_PX] = Mp[q];
+    }
+    const unsigned fl = k == 0 ? flags : mflags;
+    if (fl) atomicOr(&a.sc->flags, fl);
 }
 
 // shared -> global bulk copy by the calling thread, part of its current bulk
