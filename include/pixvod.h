@@ -108,7 +108,7 @@ typedef struct {
  *   handle stores its pixel state in the same layout (identity slot 0 holds the
  *   message from the parent, slots 1..3 are zero); its checkpoints append the
  *   node states (pixvod_save_state). The adjoint (pixvod_set_recording) returns
- *   ESTATE for a quadtree handle, and batches take grid handles only. */
+ *   ESTATE for a quadtree handle. */
 #define PIXVOD_TOPOLOGY_GRID 0
 #define PIXVOD_TOPOLOGY_QUADTREE 1
 
@@ -344,9 +344,9 @@ pixvod_status pixvod_set_backward_window(pixvod_handle* h, int32_t last_sweeps);
  *                            barrier between sweeps (blocks_per_sm resident
  *                            blocks per SM, 1..4).
  * Sequences of the quadtree topology (params.topology) batch too: under
- * PIXVOD_SCHED_BATCHED a sweep is one launch of each of the three quadtree
- * kernels (pixels, node messages, node beliefs) for all sequences; the
- * persistent schedule is for the grid only (a quadtree sweep is three dependent
+ * PIXVOD_SCHED_BATCHED a sweep is one launch of each of the two quadtree
+ * kernels (pixels and node messages, node beliefs) for all sequences; the
+ * persistent schedule is for the grid only (a quadtree sweep is two dependent
  * launches).
  * The keyframe count rule applies to the batch's frame index.
  * --------------------------------------------------------------------------- */

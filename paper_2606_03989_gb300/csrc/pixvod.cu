@@ -276,12 +276,6 @@ T* input_ptr(pixvod_handle* h, int k) {
 }
 Scalars* scalars(pixvod_handle* h) { return reinterpret_cast<Scalars*>(h->ws + h->L.off_scalars); }
 
-// the sweep's work items: tiles, or their rows in a small image
-bool row_mode(const Layout& L) {
-    return L.tiles_x * L.tiles_y <= (L.elt == 4 ? pv::row_mode_tiles<float>() : pv::row_mode_tiles<double>());
-}
-int sweep_items(const Layout& L) { return L.tiles_x * L.tiles_y * (row_mode(L) ? pv::TILE_H : 1); }
-
 template <typename T>
 pv::SeqDesc<T> seq_desc(pixvod_handle* h, const float* frame, const float* normals) {
     pv::SeqDesc<T> d{};  // every pointer not set below (the recorded-decision buffer) is null
@@ -296,7 +290,6 @@ pv::SeqDesc<T> seq_desc(pixvod_handle* h, const float* frame, const float* norma
     d.normals = normals;
     d.br = nullptr;
     d.n_tiles = h->L.tiles_x * h->L.tiles_y;
-    d.rows = row_mode(h->L) ? 1 : 0;
     return d;
 }
 
@@ -311,20 +304,48 @@ dim3 pixel_grid(const pixvod_handle* h) {
 }
 dim3 sweep_block() { return dim3(pv::SWEEP_BX, pv::SWEEP_BY); }
 
-// dynamic shared memory of the sweep kernel (above the 48 KB default for double)
+// the sweep kernel of a launch over n_tiles tiles, and its work items
+template <typename T>
+pv::SweepMode sweep_mode(int n_tiles) {
+    if (n_tiles <= pv::row_mode_tiles<T>()) return pv::SWEEP_ROWS;
+    return n_tiles > pv::stream_mode_tiles<T>() ? pv::SWEEP_STREAM : pv::SWEEP_TILES;
+}
+template <typename T>
+using SweepKernel = decltype(&pv::k_sweeps<T, pv::SWEEP_TILES>);
+template <typename T>
+SweepKernel<T> sweep_kernel(int n_tiles) {
+    switch (sweep_mode<T>(n_tiles)) {
+        case pv::SWEEP_ROWS: return &pv::k_sweeps<T, pv::SWEEP_ROWS>;
+        case pv::SWEEP_STREAM: return &pv::k_sweeps<T, pv::SWEEP_STREAM>;
+        default: return &pv::k_sweeps<T, pv::SWEEP_TILES>;
+    }
+}
+template <typename T>
+int sweep_items(int n_tiles) {
+    return sweep_mode<T>(n_tiles) == pv::SWEEP_ROWS ? n_tiles * pv::TILE_H : n_tiles;
+}
+
+// dynamic shared memory of the sweep kernels (above the 48 KB default for double)
 template <typename T>
 cudaError_t sweep_attributes() {
-    static cudaError_t once = cudaFuncSetAttribute(pv::k_sweeps<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)pv::sweep_smem_bytes<T>());
+    static cudaError_t once = [] {
+        cudaError_t e = cudaSuccess;
+        for (SweepKernel<T> k : {&pv::k_sweeps<T, pv::SWEEP_TILES>, &pv::k_sweeps<T, pv::SWEEP_STREAM>,
+                                 &pv::k_sweeps<T, pv::SWEEP_ROWS>})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)pv::sweep_smem_bytes<T>());
+        return e;
+    }();
     return once;
 }
 
 // one synchronous grid sweep: the tiles of `work` (null: of the descriptor's
 // sequence in order; from the end when `flip` is odd), reading state buffer `cur`
 template <typename T>
-void launch_sweep(const pv::SeqDesc<T>* desc, const pv::Work* work, int n_work, int cur, int flip, cudaStream_t st) {
-    launch_pdl(pv::k_sweeps<T>, dim3(n_work), sweep_block(), pv::sweep_smem_bytes<T>(), st, desc, work, n_work, 1, cur,
-               flip, pv::GridSync{nullptr, nullptr, nullptr, 0});
+void launch_sweep(const pv::SeqDesc<T>* desc, const pv::Work* work, int n_tiles, int cur, int flip, cudaStream_t st) {
+    launch_pdl(sweep_kernel<T>(n_tiles), dim3(sweep_items<T>(n_tiles)), sweep_block(), pv::sweep_smem_bytes<T>(), st,
+               desc, work, n_tiles, 1, cur, flip, pv::GridSync{nullptr, nullptr, nullptr, 0});
 }
 
 pixvod_status cuda_status(cudaError_t e) {
@@ -468,7 +489,7 @@ template <typename T>
 pixvod_status run_sweeps(pixvod_handle* h, int n) {
     pixvod_status st = cuda_status(sweep_attributes<T>());
     if (st != PIXVOD_OK) return st;
-    const int n_items = sweep_items(h->L);
+    const int n_tiles = h->L.tiles_x * h->L.tiles_y;
     for (int it = 0; it < n; ++it) {
         bool prof = h->profiling;
         if (prof) {
@@ -479,7 +500,7 @@ pixvod_status run_sweeps(pixvod_handle* h, int n) {
         if (is_quadtree(h)) {
             s = launch_qt_sweep<T>(h);
         } else {
-            launch_sweep<T>(desc_ptr<T>(h), nullptr, n_items, h->cur, h->cur, h->stream);
+            launch_sweep<T>(desc_ptr<T>(h), nullptr, n_tiles, h->cur, h->cur, h->stream);
             s = launched(h);
         }
         if (prof) {
@@ -515,7 +536,7 @@ pixvod_status run_sweeps_recorded(pixvod_handle* h, int n) {
         if (n <= 0) return PIXVOD_OK;
         pixvod_status s = cuda_status(sweep_attributes<T>());
         if (s != PIXVOD_OK) return s;
-        const int cur0 = h->cur, n_items = sweep_items(h->L);
+        const int cur0 = h->cur, n_tiles = h->L.tiles_x * h->L.tiles_y;
         std::vector<pv::SeqDesc<T>> descs(n);
         for (int c = 1; c <= n; ++c) {  // sweep c maps S_{c-1} to S_c and records its decisions
             pv::SeqDesc<T> d = seq_desc<T>(h, nullptr, nullptr);
@@ -530,7 +551,7 @@ pixvod_status run_sweeps_recorded(pixvod_handle* h, int n) {
         if (s != PIXVOD_OK) return s;
         const pv::SeqDesc<T>* dd = reinterpret_cast<const pv::SeqDesc<T>*>(h->rec_ws + R.off_desc);
         for (int c = 1; c <= n; ++c) {
-            launch_sweep<T>(dd + (c - 1), nullptr, n_items, 0, c, h->stream);
+            launch_sweep<T>(dd + (c - 1), nullptr, n_tiles, 0, c, h->stream);
             if ((s = launched(h)) != PIXVOD_OK) return s;
         }
         h->cur = cur0 ^ 1;
@@ -730,7 +751,7 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
         const int c = seg * k, len = n - c < k ? n - c : k;
         if (c + len <= first) break;
         for (int j = 1; j <= len; ++j) {
-            launch_sweep<T>(ddesc + (c + j - 1), nullptr, sweep_items(h->L), 0, j, st);
+            launch_sweep<T>(ddesc + (c + j - 1), nullptr, n_tiles, 0, j, st);
             if ((s = launched(h)) != PIXVOD_OK) return s;
         }
         for (int j = len; j >= 1 && c + j > first; --j)
@@ -1219,9 +1240,8 @@ struct pixvod_batch {
     cudaStream_t stream;
     std::vector<pixvod_handle> seq;
     char* ws;
-    size_t off_desc, off_work, off_items, off_sync;
-    int n_work;    // tiles of all sequences
-    int n_items;   // the sweep's work items (tiles, or rows of small images)
+    size_t off_desc, off_work, off_sync;
+    int n_work;
     int schedule;
     int blocks_per_sm;
     int max_blocks_per_sm;
@@ -1245,27 +1265,24 @@ namespace {
 struct BatchLayout {
     std::vector<Layout> seq;
     std::vector<size_t> off_seq;
-    size_t off_desc, off_work, off_items, off_sync, off_qtargs, off_qtoff, total;
-    int n_work, n_items;
+    size_t off_desc, off_work, off_sync, off_qtargs, off_qtoff, total;
+    int n_work;
 };
 
 BatchLayout make_batch_layout(int n, const pixvod_intrinsics* K, const pixvod_params* p) {
     BatchLayout B;
     size_t off = 0;
-    B.n_work = B.n_items = 0;
+    B.n_work = 0;
     for (int i = 0; i < n; ++i) {
         B.seq.push_back(make_layout(&K[i], p));
         B.off_seq.push_back(off);
         off += align_up(B.seq.back().total, kAlign);
         B.n_work += B.seq.back().tiles_x * B.seq.back().tiles_y;
-        B.n_items += sweep_items(B.seq.back());
     }
     B.off_desc = off;
     off += align_up((size_t)n * kDescBytes, kAlign);
     B.off_work = off;
     off += align_up((size_t)B.n_work * sizeof(pv::Work), kAlign);
-    B.off_items = off;
-    off += align_up((size_t)B.n_items * sizeof(pv::Work), kAlign);
     B.off_sync = off;
     off += kAlign;
     B.off_qtargs = B.off_qtoff = off;
@@ -1294,7 +1311,6 @@ const pv::SeqDesc<T>* descs(pixvod_batch* b) {
     return reinterpret_cast<const pv::SeqDesc<T>*>(b->ws + b->off_desc);
 }
 const pv::Work* works(pixvod_batch* b) { return reinterpret_cast<const pv::Work*>(b->ws + b->off_work); }
-const pv::Work* items(pixvod_batch* b) { return reinterpret_cast<const pv::Work*>(b->ws + b->off_items); }
 unsigned* batch_sync(pixvod_batch* b) { return reinterpret_cast<unsigned*>(b->ws + b->off_sync); }
 
 pixvod_status batch_launched(pixvod_batch* b) {
@@ -1359,7 +1375,7 @@ pixvod_status batch_sweeps(pixvod_batch* b, int n_iters, int schedule) {
         }
     } else if (schedule == PIXVOD_SCHED_BATCHED) {
         for (int it = 0; it < n_iters; ++it) {
-            launch_sweep<T>(descs<T>(b), items(b), b->n_items, cur, cur, b->stream);
+            launch_sweep<T>(descs<T>(b), works(b), b->n_work, cur, cur, b->stream);
             if ((s = batch_launched(b)) != PIXVOD_OK) return s;
             cur ^= 1;
         }
@@ -1374,12 +1390,12 @@ pixvod_status batch_sweeps(pixvod_batch* b, int n_iters, int schedule) {
             return s;
         pv::GridSync gs{sy, sy + 1, sy + 2, b->wait_limit};
         int grid = b->blocks_per_sm * b->num_sms;
-        if (grid > b->n_items) grid = b->n_items;
+        if (grid > sweep_items<T>(b->n_work)) grid = sweep_items<T>(b->n_work);
         const pv::SeqDesc<T>* d = descs<T>(b);
-        const pv::Work* w = items(b);
-        int n_work = b->n_items, cur0 = cur;
+        const pv::Work* w = works(b);
+        int n_work = b->n_work, cur0 = cur;
         void* args[] = {(void*)&d, (void*)&w, (void*)&n_work, (void*)&n_iters, (void*)&cur0, (void*)&cur0, (void*)&gs};
-        s = cuda_status(cudaLaunchCooperativeKernel((const void*)pv::k_sweeps<T>, dim3(grid), sweep_block(),
+        s = cuda_status(cudaLaunchCooperativeKernel((const void*)sweep_kernel<T>(n_work), dim3(grid), sweep_block(),
                                                     args, pv::sweep_smem_bytes<T>(), b->stream));
         b->launches++;
         if (s != PIXVOD_OK) return s;
@@ -1533,8 +1549,6 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
     b->ws = static_cast<char*>(d_workspace);
     b->off_desc = B.off_desc;
     b->off_work = B.off_work;
-    b->off_items = B.off_items;
-    b->n_items = B.n_items;
     b->off_sync = B.off_sync;
     b->off_qtargs = B.off_qtargs;
     b->off_qtoff = B.off_qtoff;
@@ -1583,13 +1597,13 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
     if (s == PIXVOD_OK) {
         int m = 0;
         s = cuda_status(p->precision == 64
-                            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, pv::k_sweeps<double>,
+                            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, sweep_kernel<double>(B.n_work),
                                                                             pv::SWEEP_THREADS,
                                                                             pv::sweep_smem_bytes<double>())
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, pv::k_sweeps<float>,
+                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, sweep_kernel<float>(B.n_work),
                                                                             pv::SWEEP_THREADS,
                                                                             pv::sweep_smem_bytes<float>()));
-        // the persistent schedule runs grid sequences (a quadtree sweep is three
+        // the persistent schedule runs grid sequences (a quadtree sweep is two
         // dependent launches)
         b->max_blocks_per_sm = coop && !b->qt ? (m < 4 ? m : 4) : 0;
         b->blocks_per_sm = b->max_blocks_per_sm;
@@ -1609,18 +1623,12 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
         if (s == PIXVOD_OK) s = cuda_status(cudaStreamSynchronize(b->stream));  // eye outlives the copies
     }
     if (s == PIXVOD_OK) {
-        std::vector<pv::Work> w, items;
+        std::vector<pv::Work> w;
         w.reserve(B.n_work);
-        items.reserve(B.n_items);
-        for (int i = 0; i < n; ++i) {
+        for (int i = 0; i < n; ++i)
             for (int t = 0; t < B.seq[i].tiles_x * B.seq[i].tiles_y; ++t) w.push_back(pv::Work{i, t});
-            for (int t = 0; t < sweep_items(B.seq[i]); ++t) items.push_back(pv::Work{i, t});
-        }
         s = cuda_status(cudaMemcpyAsync(b->ws + b->off_work, w.data(), w.size() * sizeof(pv::Work),
                                         cudaMemcpyHostToDevice, b->stream));
-        if (s == PIXVOD_OK)
-            s = cuda_status(cudaMemcpyAsync(b->ws + b->off_items, items.data(), items.size() * sizeof(pv::Work),
-                                            cudaMemcpyHostToDevice, b->stream));
         if (s == PIXVOD_OK) s = p->precision == 64 ? upload_descs<double>(b) : upload_descs<float>(b);
         if (s == PIXVOD_OK && b->qt) s = p->precision == 64 ? upload_qt<double>(b) : upload_qt<float>(b);
         if (s == PIXVOD_OK) s = cuda_status(cudaStreamSynchronize(b->stream));

@@ -24,16 +24,29 @@ struct SeqDesc {
     const float* normals;
     unsigned char* br;     // decisions of the sweep, recorded for the adjoint (or null)
     int n_tiles;
-    int rows;              // the sweep's work items are rows of tiles (4 tile + row), not tiles
 };
 
-// An image of at most this many tiles is swept by rows (sweep_row): two tiles per
-// SM in FP32 (measured: faster at 280 tiles, slower at 384), half a tile in FP64
-// (the rows then fit on the SMs at once; faster at 24 and 48 tiles, slower at 96).
+// A launch over at most this many tiles (of one image, or of a batch together) sweeps
+// them by rows (sweep_row): two tiles per SM in FP32 (measured: faster at 280 tiles,
+// slower at 384), half a tile in FP64 (the rows then fit on the SMs at once; faster at
+// 24 and 48 tiles, slower at 96).
 template <typename T>
 constexpr int row_mode_tiles() {
     return sizeof(T) == 4 ? 304 : 76;
 }
+
+// A launch over more tiles than this marks the new state's plane stores to leave L2
+// first: one wave of tiles in FP32 (4 blocks on 152 SMs), whose two buffers (94 MB)
+// L2 still holds in the next sweep. Larger states do not stay anyway, and what is
+// evicted is then rather the output than the neighbours' planes still to be read: a
+// sweep at 320x240 20.5 and 21.1 us without and with, 333x251 30.9 and 30.5, 512x384
+// 58.7 and 57.4, 640x480 86.5 and 85.2, 2048x1536 821 and 796; FP64 the same to 0.2 %.
+template <typename T>
+constexpr int stream_mode_tiles() {
+    return sizeof(T) == 4 ? 608 : 304;
+}
+
+enum SweepMode { SWEEP_TILES, SWEEP_STREAM, SWEEP_ROWS };
 
 struct Work {
     int seq;
@@ -55,7 +68,6 @@ __device__ __forceinline__ SweepArgs<T> seq_args(const SeqDesc<T>& d, int cur) {
     a.m_y = d.in_planes[5];
     a.sc = d.sc;
     a.br = d.br;
-    a.rows = d.rows;
     return a;
 }
 
@@ -100,52 +112,58 @@ __device__ __forceinline__ bool grid_sync(const GridSync& gs) {
     return ok_sh != 0;
 }
 
-// Synchronous sweeps over a list of (sequence, tile or row of a tile) work items. This one kernel
-// serves every schedule, so a tile's arithmetic is the same machine code however
-// the work is launched (and the results do not depend on the schedule):
-//  - one sweep per launch, one block per work item (n_iters == 1, grid == n_work);
+// Synchronous sweeps over a list of (sequence, tile) work items; with ROWS each item
+// is cut into its TILE_H rows, a block each. A pixel is computed by the same functions
+// in the same order either way, and each kernel serves every schedule, so the
+// results do not depend on how the work is launched:
+//  - one sweep per launch, one block per tile or row (n_iters == 1);
 //  - n_iters sweeps in one cooperative launch: blocks stride over the work list
 //    and meet at a grid barrier between sweeps. A sweep's stores (generic proxy)
 //    are then read by the next sweep's bulk copies (async proxy) on other SMs, so
 //    every thread fences the two proxies after its tile, before the barrier
 //    publishes the stores.
-// work == nullptr stands for the tiles of sequence 0 in order.
-template <typename T>
+// work == nullptr stands for the tiles of sequence 0 in order. ROWS is a kernel of its
+// own: with both paths in one, 256x256 took 19.3 us a sweep instead of 18.9 and
+// 2048x1536 837 instead of 821.
+template <typename T, SweepMode MODE>
 __global__ void __launch_bounds__(SWEEP_THREADS, sizeof(T) == 4 ? 4 : 2) k_sweeps(const SeqDesc<T>* __restrict__ seqs,
-                                                             const Work* __restrict__ work, int n_work,
+                                                             const Work* __restrict__ work, int n_tiles,
                                                              int n_iters, int cur0, int flip0,
                                                              GridSync gs) {
-    // msg[p * TILE_PX + tid]: a tile's 108 identity-message planes, bulk-copied in
-    // at the start of the tile (the old messages), overwritten in place by the
-    // damped new ones
+    // msg[p * TILE_PX + tid]: a tile's 84 message Lambda planes, bulk-copied in at the
+    // start of the tile (the old messages), overwritten in place by the damped new
+    // ones; by rows, the four directions' messages of the row
+    constexpr bool ROWS = MODE == SWEEP_ROWS;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
-    if (threadIdx.x == 0 && threadIdx.y == 0) mbar_init(&bar, 1);
-    __syncthreads();
+    if (!ROWS) {
+        if (threadIdx.x == 0 && threadIdx.y == 0) mbar_init(&bar, 1);
+        __syncthreads();
+    }
     pdl_wait();
     T* msg = reinterpret_cast<T*>(smem_raw);
     unsigned parity = 0;
+    const int n_work = ROWS ? n_tiles * TILE_H : n_tiles;
     for (int it = 0; it < n_iters; ++it) {
         const int cur = (cur0 + it) & 1;
         // every other sweep takes the work from its end: what the previous sweep wrote
         // last is what L2 still holds
         const bool flip = (flip0 + it) & 1;
         for (int k = blockIdx.x; k < n_work; k += gridDim.x) {
-            const int w = flip ? n_work - 1 - k : k;
-            const Work wk = work ? work[w] : Work{0, w};
+            const int w = flip ? n_work - 1 - k : k, item = ROWS ? w / TILE_H : w;
+            const Work wk = work ? work[item] : Work{0, item};
             const SweepArgs<T> a = seq_args(seqs[wk.seq], cur);
-            const int tile = a.rows ? wk.tile / TILE_H : wk.tile, tx = tile % a.g.tiles_x, ty = tile / a.g.tiles_x;
-            if (a.rows) {
-                sweep_row(a, tx, ty, wk.tile % TILE_H, msg, it + 1 == n_iters);
-                __syncthreads();
-                continue;
+            const int tx = wk.tile % a.g.tiles_x, ty = wk.tile / a.g.tiles_x;
+            if (ROWS) {
+                sweep_row(a, tx, ty, w % TILE_H, msg, it + 1 == n_iters);
+            } else {
+                // a tile whose bulk copy never arrived ends the block's work for the
+                // launch: the mbarrier's phase no longer matches `parity`, and the copy
+                // may still be writing `msg`
+                if (!sweep_tile<MODE == SWEEP_STREAM>(a, tx, ty, msg, &bar, parity, it + 1 == n_iters)) return;
+                parity ^= 1u;
+                if (n_iters > 1) asm volatile("fence.proxy.async.global;" ::: "memory");
             }
-            // a tile whose bulk copy never arrived ends the block's work for the
-            // launch: the mbarrier's phase no longer matches `parity`, and the copy
-            // may still be writing `msg`
-            if (!sweep_tile(a, tx, ty, msg, &bar, parity, it + 1 == n_iters)) return;
-            parity ^= 1u;
-            if (n_iters > 1) asm volatile("fence.proxy.async.global;" ::: "memory");
             __syncthreads();
         }
         if (it + 1 < n_iters && !grid_sync(gs)) return;

@@ -110,7 +110,6 @@ struct SweepArgs {
     // when set, each pixel's discrete decisions of this sweep (BR_* bits) are
     // written here (tile-major pixel index), for the adjoint
     unsigned char* br;
-    int rows;  // work items are rows of tiles (sweep_row), not tiles
 };
 
 
@@ -283,6 +282,16 @@ template <typename T>
 __device__ __forceinline__ T ld_state(const T* p) {
     return __ldcg(p);
 }
+// A product that no addition after it is fused with (the sweep by tiles and by rows
+// then round alike)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+// Store of the new state; STREAM: marked to leave L2 first (st.global.cs)
+template <bool STREAM, typename T>
+__device__ __forceinline__ void st_state(T* p, T x) {
+    if (STREAM) __stcs(p, x);
+    else *p = x;
+}
 
 // Thread block of the sweep kernel: one state tile (32 x 4 pixels), one thread
 // per pixel; 4 blocks per SM (43 KB of shared memory and at most 128 registers
@@ -312,8 +321,8 @@ constexpr size_t sweep_smem_bytes() {
 
 // a1: photometric factor (Eqs. 2, 3) of pixel (u, v), input-plane index i, at the
 // mean (qi, t, d)
-template <typename T>
-__device__ __forceinline__ void photometric_factor(const SweepArgs<T>& a, int i, int u, int v, const T* qi, const T* t,
+template <typename T, typename Args>
+__device__ __forceinline__ void photometric_factor(const Args& a, int i, int u, int v, const T* qi, const T* t,
                                                    T d, T* J, T& alpha, T& rph, unsigned char& br, unsigned& flags) {
     const Geometry<T>& g = a.g;
     const Factors<T>& F = a.f;
@@ -515,7 +524,7 @@ __device__ __forceinline__ void depth_marginals(T md, T alpha, T Jd, T qv, T* sb
 // The calling thread's pixel of the sweep over tile (tx, ty): everything but the
 // store of the identity messages' Lambda, which are left in `msg`. False if the
 // tile's bulk copy never arrived (FLAG_TIMEOUT is set).
-template <typename T>
+template <bool STREAM, typename T>
 __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int ty, T* msg, uint64_t* bar,
                                             unsigned parity) {
     const int tid = threadIdx.y * SWEEP_BX + threadIdx.x;
@@ -541,9 +550,9 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
     // --- priors (Eq. 4 with identity Jacobian; log-depth prior) ---
     T eb[7];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) eb[k] = -(F.lam_P * xi[k]);
+    for (int k = 0; k < 6; ++k) eb[k] = -mul_rn(F.lam_P, xi[k]);
     T md = F.lam_Z;
-    eb[6] = -(F.lam_Z * (d - T(a.sc->d_prior)));
+    eb[6] = -mul_rn(F.lam_Z, d - T(a.sc->d_prior));
 
     T alpha, rph, J[7];
     unsigned char br;
@@ -624,23 +633,23 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
         T xn[6];
         se3_update(qi, t, tau, xn);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) Di[q * TILE_PX] = xn[q];
-        Di[6 * TILE_PX] = d + tau[6];
+        for (int q = 0; q < 6; ++q) st_state<STREAM>(&Di[q * TILE_PX], xn[q]);
+        st_state<STREAM>(&Di[6 * TILE_PX], d + tau[6]);
     }
     {
         T sb, s;
         depth_marginals(md, alpha, J[6], qv, &sb, &s);
 #pragma unroll
-        for (int q = 0; q < 21; ++q) Di[(PL_MP + q) * TILE_PX] = Mp[q];
+        for (int q = 0; q < 21; ++q) st_state<STREAM>(&Di[(PL_MP + q) * TILE_PX], Mp[q]);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) Di[(PL_U + q) * TILE_PX] = sb * J[q];
-        Di[PL_S * TILE_PX] = s;
+        for (int q = 0; q < 6; ++q) st_state<STREAM>(&Di[(PL_U + q) * TILE_PX], sb * J[q]);
+        st_state<STREAM>(&Di[PL_S * TILE_PX], s);
     }
     // messages, projected: eta <- eta - Lambda tau
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        Di[(PL_NM + 2 * k) * TILE_PX] = nl[k];
-        Di[(PL_NM + 2 * k + 1) * TILE_PX] = ne[k] - nl[k] * tau[6];
+        st_state<STREAM>(&Di[(PL_NM + 2 * k) * TILE_PX], nl[k]);
+        st_state<STREAM>(&Di[(PL_NM + 2 * k + 1) * TILE_PX], ne[k] - nl[k] * tau[6]);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -650,7 +659,7 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
             T e = en[6 * k + r];
 #pragma unroll
             for (int c = 0; c < 6; ++c) e -= mb[pidx(r, c) * TILE_PX] * tau[c];
-            Di[(PL_ID + ID_STRIDE * k + LAM + r) * TILE_PX] = e;
+            st_state<STREAM>(&Di[(PL_ID + ID_STRIDE * k + LAM + r) * TILE_PX], e);
         }
     }
     if (flags) atomicOr(&a.sc->flags, flags);
@@ -741,8 +750,8 @@ __device__ __forceinline__ void sweep_row(const SweepArgs<T>& a, int tx, int ty,
         Mp[q] = y;
     }
 #pragma unroll
-    for (int q = 0; q < 6; ++q) eb[q] = -(F.lam_P * xi[q]);
-    eb[6] = -(F.lam_Z * (d - T(a.sc->d_prior)));
+    for (int q = 0; q < 6; ++q) eb[q] = -mul_rn(F.lam_P, xi[q]);
+    eb[6] = -mul_rn(F.lam_Z, d - T(a.sc->d_prior));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const T* sj = msg + j * ROW_VALUES * TILE_W + x;
@@ -823,7 +832,7 @@ __device__ __forceinline__ void bulk_wait_s2g(bool last_sweep) {
 // false (to every thread) when the tile's bulk copy did not arrive within the
 // bounded wait: nothing of the tile was stored, FLAG_TIMEOUT is set, and the
 // block must take no further tile in this launch.
-template <typename T>
+template <bool STREAM, typename T>
 __device__ __forceinline__ bool sweep_tile(const SweepArgs<T>& a, int tx, int ty, T* msg, uint64_t* bar,
                                            unsigned parity, bool last_sweep) {
     const int tid = threadIdx.y * SWEEP_BX + threadIdx.x;
@@ -838,7 +847,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs<T>& a, int tx, int ty
             bulk_copy_g2s(msg + LAM * k * TILE_PX, a.in + tile * TILE_WORDS + (PL_ID + ID_STRIDE * k) * TILE_PX, bytes,
                           bar);
     }
-    const bool ok = sweep_pixel(a, tx, ty, msg, bar, parity);
+    const bool ok = sweep_pixel<STREAM>(a, tx, ty, msg, bar, parity);
     // the messages written to shared memory (generic proxy) are read by
     // the bulk copy (async proxy): fence, then gather the block; a tile whose
     // messages never arrived is not stored

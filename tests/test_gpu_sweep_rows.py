@@ -1,6 +1,6 @@
 """The sweep by rows (images of few tiles) and by tiles, on both sides of the rule
 that chooses between them and at ragged sizes: one sweep against the oracle, and
-batches that mix the two against their sequences tracked alone, bit for bit."""
+batches swept by tiles or by rows against their sequences tracked alone, bit for bit."""
 import numpy as np
 import pytest
 
@@ -32,8 +32,9 @@ def test_one_sweep_on_both_sides_of_the_rule(prec, size, tiles):
                     sample_pixels(h, w, min(60, w * h), prec))
 
 
-@pytest.mark.parametrize("prec,sizes", [(32, [(608, 63), (609, 61), (70, 45)]), (64, [(127, 74), (129, 61), (33, 17)])])
-def test_a_batch_of_both_matches_its_sequences(prec, sizes):
+@pytest.mark.parametrize("prec,sizes", [(32, [(608, 63), (609, 61), (70, 45)]), (32, [(70, 45), (320, 61), (31, 3)]),
+                                         (64, [(127, 74), (129, 61), (33, 17)]), (64, [(33, 17), (65, 35)])])
+def test_a_batch_matches_its_sequences(prec, sizes):
     seqs = [synth.realistic(60 + i, 3, w, h) for i, (w, h) in enumerate(sizes)]
     frames = [[torch.from_numpy(s.frame(k)).to(DEV) for k in range(3)] for s in seqs]
     normals = [torch.from_numpy(s.normals(0)).to(DEV) for s in seqs]
