@@ -641,7 +641,9 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
     double* dparam = misc;                                                        // 3 doubles
     unsigned long long* mism = reinterpret_cast<unsigned long long*>(misc + 4);  // 1
     unsigned* fl = reinterpret_cast<unsigned*>(misc + 5);                        // flags, max nodes
-    double* scale = misc + 8;  // exponent of the adjoint state's units and the pass's factors (6 doubles)
+    pv::AdjScale* scale = reinterpret_cast<pv::AdjScale*>(misc + 8);  // factors of the even and the odd passes
+    unsigned long long* adj_max = reinterpret_cast<unsigned long long*>(scale + 2);
+    unsigned* ticket = reinterpret_cast<unsigned*>(adj_max + 1);
     pixvod_status s = cuda_status(sweep_attributes<T>());
     if (s == PIXVOD_OK) s = cuda_status(cudaMemsetAsync(dIs, 0, npx * sizeof(double), st));
     if (s == PIXVOD_OK) s = cuda_status(cudaMemsetAsync(dIt, 0, npx * sizeof(double), st));
@@ -703,7 +705,7 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
     A.tape.adj = reinterpret_cast<double*>(rw + R.off_tadj);
     A.tape.cap = kTapeCap;
     A.tape.n_slots = R.slots;
-    A.scale = scale;
+    A.adj_max = adj_max;
     const size_t adj_elems = (size_t)n_tiles * pv::TILE_WORDS;
     const size_t adj_used = adj_elems * (adj64 ? sizeof(double) : sizeof(float));  // of the FP64-sized buffers
     // the prior mean of the segment the frame was tracked in
@@ -713,6 +715,7 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
     if (s != PIXVOD_OK) return s;
     A.d_prior = d_prior;
     int a = 0;  // adjoint buffer holding the adjoint of the later state
+    int passes = 0;
     // sweeps first+1 .. n are differentiated; the state after sweep `first` is a constant
     const int first = h->rec_window > 0 && h->rec_window < n ? n - h->rec_window : 0;
     // the reverse pass of one sweep S_in -> S_out with its recorded decisions
@@ -729,12 +732,15 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
             if ((r = cuda_status(pv::launch_adjoint_sweep(A, R.slots / pv::ad::ADJ_THREADS, st))) != PIXVOD_OK)
                 return r;
         } else {
-            // rescale by a power of two: max |adj_out| and the factors (which also
-            // zeroes adj_in), then the pass
-            h->launches += 1 + pv::ADJOINT_HW_LAUNCHES;
-            if ((r = cuda_status(pv::launch_adjoint_absmax(adj[a], adj[a ^ 1], adj_elems, adj64 ? 1 : 0, scale,
-                                                           st))) != PIXVOD_OK)
-                return r;
+            A.scale = scale + (passes & 1);
+            A.scale_next = scale + (~passes & 1);
+            h->launches += pv::ADJOINT_HW_LAUNCHES;
+            if (passes++ == 0) {
+                h->launches++;
+                if ((r = cuda_status(pv::launch_adjoint_absmax(adj[a], adj_elems, adj64 ? 1 : 0, scale, adj_max, ticket,
+                                                               st))) != PIXVOD_OK)
+                    return r;
+            }
             if ((r = cuda_status(pv::launch_adjoint_hw(A, n_tiles, rw + R.off_scr, st))) != PIXVOD_OK) return r;
         }
         a ^= 1;

@@ -60,7 +60,9 @@ struct HwArgs {
     double* dI_t;
     double* dparam;
     unsigned long long* mismatch;
-    const double* scale;  // [2], [3] and the two ints at [5]: the pass's factors (k_adjoint_absmax)
+    const AdjScale* scale;
+    AdjScale* scale_next;
+    unsigned long long* adj_max;
 };
 
 template <typename T>
@@ -102,6 +104,8 @@ HwArgs<T> hw_args(const AdjArgs& A) {
     h.dparam = A.dparam;
     h.mismatch = A.mismatch;
     h.scale = A.scale;
+    h.scale_next = A.scale_next;
+    h.adj_max = A.adj_max;
     return h;
 }
 
@@ -130,9 +134,10 @@ struct KernelIO {
     size_t si, sj[DIR ? 1 : 4];
     int tx[4], ty[4];
     T Is, tapv[12];
-    T in_scale;        // 2^-e: adj_out is read in units of 2^(E + e)
-    int out_exp;       // E + e: the FP64 gradients' factor is 2^out_exp
+    T in_scale;        // adj_out is read times this
+    int out_exp;       // the FP64 gradients' factor is 2^out_exp
     double out_scale;
+    mutable T ymax;    // largest |adj_out| read (finite), scaled
     T dIs, lamD, isD, lamN;  // one value each in a pixel's pass
 
     __device__ size_t nbi(int k) const { return DIR ? sj[0] : sj[k]; }
@@ -142,7 +147,11 @@ struct KernelIO {
     __device__ T nb(int k, int q) const { return __ldg(Sin + nbi(k) + nb_plane(q, k) * TILE_PX); }
     __device__ T I_s() const { return Is; }
     __device__ T tap(int q) const { return tapv[q]; }
-    __device__ T ybar(int q) const { return __ldcg(Ao + si + q * TILE_PX) * in_scale; }
+    __device__ T ybar(int q) const {
+        const T y = __ldcg(Ao + si + q * TILE_PX) * in_scale, b = v_abs(y);
+        if (b > ymax && v_finite(b)) ymax = b;
+        return y;
+    }
     // the stages' scratch (scr_in, scr_out: the pixel's planes)
     const T* scr_in;
     T* scr_out;
@@ -219,15 +228,16 @@ __device__ bool pixel_context(const HwArgs<T>& A, int tile, int lane, int k, hw:
     io.scr_in = nullptr;
     io.scr_out = nullptr;
     io.dIs = io.lamD = io.isD = io.lamN = T(0);
+    io.ymax = T(0);
     // The adjoint state is rescaled by a power of two before every pass: the
     // unrolled derivative can grow by many orders of magnitude over the sweeps,
     // beyond the float range, while the pass is linear in its input.
     if constexpr (sizeof(T) == 4)
-        io.in_scale = __ldcg(reinterpret_cast<const float*>(A.scale + 5));
+        io.in_scale = __ldcg(&A.scale->in32);
     else
-        io.in_scale = __ldcg(A.scale + 2);
-    io.out_scale = __ldcg(A.scale + 3);
-    io.out_exp = __ldcg(reinterpret_cast<const int*>(A.scale + 5) + 1);
+        io.in_scale = __ldcg(&A.scale->in);
+    io.out_scale = __ldcg(&A.scale->out);
+    io.out_exp = __ldcg(&A.scale->E32);
     c.u = T(u);
     c.v = T(v);
     c.W = W;
@@ -322,8 +332,8 @@ __device__ __forceinline__ void check_vec(const T* y, const T* scale, const T* r
     for (int r = 0; r < 6; ++r) check_value(y[r], scale[r] > b ? scale[r] : b, rv[r], mm);
 }
 
-// the block's largest difference to *mismatch (every thread calls it)
-template <typename T>
+// the block's largest mm to *mismatch (every thread calls it, once in a kernel per WHICH)
+template <int WHICH = 0, typename T>
 __device__ __forceinline__ void check_block_max(T mm, unsigned long long* mismatch) {
     __shared__ T wm[TILE_PX / 32];
     for (int o = 16; o > 0; o >>= 1) {
@@ -349,6 +359,15 @@ __global__ void __launch_bounds__(TILE_PX) k_adjoint_fwd(const HwArgs<T> A, T* _
     pdl_wait();
     const int tile = blockIdx.x, k = threadIdx.x & 3;
     const int lane = blockIdx.y * TILE_W + (threadIdx.x >> 2);
+    {  // adj_in, a quarter of the tile's words per block
+        struct alignas(16) V {
+            T x[16 / sizeof(T)];
+        };
+        constexpr int n = TILE_WORDS / TILE_H * (int)sizeof(T) / 16;
+        static_assert(TILE_WORDS % (TILE_H * 16 / sizeof(T)) == 0, "whole 16-byte words");
+        V* z = reinterpret_cast<V*>(A.Ai + (size_t)tile * TILE_WORDS + blockIdx.y * (TILE_WORDS / TILE_H));
+        for (int i = threadIdx.x; i < n; i += TILE_PX) z[i] = V{};
+    }
     KernelIO<T, true> io;
     hw::PixCtx<T> c;
     int u, v;
@@ -409,6 +428,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? PV_ADJ_MAIN_BLOCKS :
     const int tile = blockIdx.x, lane = threadIdx.x;
     __shared__ double red[3][TILE_PX / 32];
     double sums[3] = {0.0, 0.0, 0.0};
+    T ymax = T(0);
     KernelIO<T, false> io;
     hw::PixCtx<T> c;
     int u, v;
@@ -466,6 +486,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? PV_ADJ_MAIN_BLOCKS :
         sums[0] = scaled_double(io.lamD, io.out_exp, io.out_scale);
         sums[1] = scaled_double(io.isD, io.out_exp, io.out_scale);
         sums[2] = scaled_double(io.lamN, io.out_exp, io.out_scale);
+        ymax = io.ymax;
     }
     // the block's sums (as 384 FP64 atomics on shared memory they were a
     // compare-and-swap loop per lane)
@@ -482,6 +503,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? PV_ADJ_MAIN_BLOCKS :
         for (int w = 0; w < TILE_PX / 32; ++w) x += red[lane][w];
         if (x != 0.0) atomicAdd(A.dparam + lane, x);
     }
+    check_block_max(ymax, A.adj_max);
     pdl_trigger();
 }
 
@@ -499,7 +521,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? 4 : 1) k_adjoint_dir
     hw::PixCtx<T> c;
     int u, v;
     bool has = false;
-    T mm = T(0);
+    T mm = T(0), ymax = T(0);
     if (pixel_context(A, tile, lane, k, c, io, &u, &v, &has) && has) {
         T* sp = scr + (size_t)tile * SCR_WORDS + lane;
         io.scr_in = sp;
@@ -538,17 +560,33 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? 4 : 1) k_adjoint_dir
         hw::identity_vjp(io, c, k, R, t, f, Lb, eb, Rb, tb);
         for (int q = 0; q < 9; ++q) atomicAdd(sp + (SCR_MAIN + hw::MO_RB + q) * TILE_PX, Rb[q]);
         for (int q = 0; q < 3; ++q) atomicAdd(sp + (SCR_MAIN + hw::MO_TB + q) * TILE_PX, tb[q]);
+        ymax = io.ymax;
     }
     check_block_max(mm, A.mismatch);
+    check_block_max<1>(ymax, A.adj_max);
     pdl_trigger();
 }
 
+// a pass's factors: e = ilogb(max) (0 where there is none) on top of the units E
+__device__ __forceinline__ void set_scale(AdjScale* s, double E, double max) {
+    int e = (max > 0.0 && isfinite(max)) ? ilogb(max) : 0;
+    if (e < -126) e = -126;  // 2^-e stays a float
+    s->E = E + double(e);
+    s->in = ldexp(1.0, -e);
+    s->out = ldexp(1.0, (int)s->E);
+    s->in32 = (float)s->in;
+    s->E32 = (int)s->E;
+}
+
 // Pose stage (last): the pixel's xi adjoint from the (R, t) adjoints of its Exp,
-// and the recompute check of what the main stage left (SCR_CHK).
+// the recompute check of what the main stage left (SCR_CHK), and the next pass's
+// factors.
 template <typename T>
 __global__ void __launch_bounds__(TILE_PX) k_adjoint_pose(const HwArgs<T> A, const T* __restrict__ scr) {
     pdl_wait();
     const int tile = blockIdx.x, lane = threadIdx.x;
+    if (tile == 0 && lane == 0)
+        set_scale(A.scale_next, __ldcg(&A.scale->E), __longlong_as_double((long long)atomicExch(A.adj_max, 0ull)));
     KernelIO<T, true> io;
     hw::PixCtx<T> c;
     int u, v;
@@ -602,20 +640,14 @@ __device__ __forceinline__ void absmax_acc(double2 x, double& m) {
     for (int q = 0; q < 2; ++q)
         if (isfinite(v[q]) && v[q] > m) m = v[q];
 }
-// Also zeroes z (the next pass's adj_in), and its last block prepares the pass's
-// scale factors: with e = ilogb(max), scale[0] += e (the units of the adjoint
-// state after the pass), scale[2] = 2^-e, scale[3] = 2^scale[0], at scale[5] 2^-e as a
-// float and scale[0] as an int; scale[1] (the maximum) and the ticket are 0 again for the next pass.
+// Its last block sets the first pass's factors.
 template <typename T, typename V>
-__global__ void k_adjoint_absmax(const V* __restrict__ a, V* __restrict__ z, size_t nv, double* __restrict__ scale,
-                                 unsigned* __restrict__ ticket) {
+__global__ void k_adjoint_absmax(const V* __restrict__ a, size_t nv, AdjScale* __restrict__ scale,
+                                 unsigned long long* __restrict__ mx, unsigned* __restrict__ ticket) {
     pdl_wait();
-    unsigned long long* mx = reinterpret_cast<unsigned long long*>(scale + 1);
     T m = T(0);
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (size_t)gridDim.x * blockDim.x) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += (size_t)gridDim.x * blockDim.x)
         absmax_acc(__ldcg(a + i), m);
-        z[i] = V{};
-    }
     for (int o = 16; o > 0; o >>= 1) {
         const T y = __shfl_xor_sync(0xffffffffu, m, o);
         m = y > m ? y : m;
@@ -625,13 +657,7 @@ __global__ void k_adjoint_absmax(const V* __restrict__ a, V* __restrict__ z, siz
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(ticket, 1u) == gridDim.x - 1) {
         __threadfence();
-        const double v = __longlong_as_double((long long)atomicExch(mx, 0ull));
-        const int e = (v > 0.0 && isfinite(v)) ? ilogb(v) : 0;
-        scale[0] += double(e);
-        scale[2] = ldexp(1.0, -e);
-        scale[3] = ldexp(1.0, (int)scale[0]);
-        reinterpret_cast<float*>(scale + 5)[0] = (float)scale[2];
-        reinterpret_cast<int*>(scale + 5)[1] = (int)scale[0];
+        set_scale(scale, 0.0, __longlong_as_double((long long)atomicExch(mx, 0ull)));
         *ticket = 0u;
     }
     pdl_trigger();
@@ -647,15 +673,15 @@ static int stride_blocks() {
     return (sms > 0 ? sms : 152) * 8;
 }
 
-cudaError_t launch_adjoint_absmax(const void* a, void* z, size_t n, int adj64, double* scale, cudaStream_t st) {
+cudaError_t launch_adjoint_absmax(const void* a, size_t n, int adj64, AdjScale* scale, unsigned long long* max,
+                                  unsigned* ticket, cudaStream_t st) {
     const dim3 blocks(stride_blocks());
-    unsigned* ticket = reinterpret_cast<unsigned*>(scale + 4);
     if (adj64)
-        launch_pdl(k_adjoint_absmax<double, double2>, blocks, dim3(256), 0, st, static_cast<const double2*>(a),
-                   static_cast<double2*>(z), n / 2, scale, ticket);
+        launch_pdl(k_adjoint_absmax<double, double2>, blocks, dim3(256), 0, st, static_cast<const double2*>(a), n / 2,
+                   scale, max, ticket);
     else
-        launch_pdl(k_adjoint_absmax<float, float4>, blocks, dim3(256), 0, st, static_cast<const float4*>(a),
-                   static_cast<float4*>(z), n / 4, scale, ticket);
+        launch_pdl(k_adjoint_absmax<float, float4>, blocks, dim3(256), 0, st, static_cast<const float4*>(a), n / 4,
+                   scale, max, ticket);
     return cudaGetLastError();
 }
 

@@ -27,6 +27,22 @@ constexpr unsigned FLAG_TAPE_FULL = 0x8u;  // a pixel's tape overflowed: its gra
 // FP64 when state64 is set, FP32 otherwise. The adjoint states are FP64 for the
 // tape kernel and in the state's precision for the hand-written one; the
 // gradients of the inputs and factor weights are FP64.
+// Rescaling of the adjoint state by a power of two: a pass reads adj_out, in units
+// of 2^(E - e), times 2^-e, so that its adj_in and its gradients are in units of 2^E.
+// For the first pass e = ilogb(max |adj_out|) (launch_adjoint_absmax); each pass
+// leaves the next one's factors, e = ilogb of the largest value it read itself,
+// scaled. That is one pass behind: a pass reads values up to twice the growth of the
+// adjoint over one sweep (6x on the benchmark's frames), far inside the float range,
+// and no pass of its own over the 151 planes is needed (19.5 us of 173 per reverse
+// sweep at 320x240 in FP32).
+struct AdjScale {
+    double E;
+    double in;      // 2^-e
+    double out;     // 2^E
+    float in32;     // in
+    int E32;        // E
+};
+
 struct AdjArgs {
     Geometry<double> g;
     int state64;
@@ -49,11 +65,11 @@ struct AdjArgs {
     unsigned* max_nodes;           // longest tape of a pixel
     unsigned* flags;
     ad::TapeCtl tape;
-    // hand-written pass (scale[0..5], zero before the first): the adjoint state
-    // holds values in units of 2^E, E = scale[0]; the pass reads adj_out times
-    // scale[2] = 2^-e with e = ilogb(max |adj_out|), so its adj_in is in units of
-    // scale[3] = 2^(E + e) (launch_adjoint_absmax sets both and adds e to E)
-    double* scale;
+    // hand-written pass: the factors of this pass and of the one after it, and the
+    // largest |adj_out| this pass reads (as bits)
+    AdjScale* scale;
+    AdjScale* scale_next;
+    unsigned long long* adj_max;
 };
 
 // adjoint of one sweep by the reverse-mode tape (FP64), `blocks` blocks of
@@ -61,7 +77,7 @@ struct AdjArgs {
 cudaError_t launch_adjoint_sweep(const AdjArgs& A, int blocks, cudaStream_t st);
 // adjoint of one sweep by the hand-written reverse pass, in the state's
 // precision, as ADJOINT_HW_LAUNCHES launches: per pixel and direction (the
-// damped identity messages summed over the directions), per pixel (the update and
+// damped identity messages summed over the directions; also zeroes adj_in), per pixel (the update and
 // the reverse pass of everything but the identity messages), per pixel and
 // direction (the identity messages' reverse pass), per pixel (the pose), each with
 // its part of the recompute check; `scratch` (adjoint_scratch_bytes) carries values
@@ -74,9 +90,10 @@ cudaError_t launch_adjoint_hw(const AdjArgs& A, int n_tiles, void* scratch, cuda
 // (adj64) or FP32
 cudaError_t launch_adjoint_seed(const AdjArgs& A, const double* grad_xi, const double* grad_invdepth, void* adj,
                                 int adj64, cudaStream_t st);
-// the scale factors of the pass that reads a (AdjArgs::scale), from max |a[i]| over
-// n elements (finite values), and z[i] = 0 over the same n elements (its adj_in)
-cudaError_t launch_adjoint_absmax(const void* a, void* z, size_t n, int adj64, double* scale, cudaStream_t st);
+// the factors of the first pass, which reads a, from max |a[i]| over n elements
+// (finite values); `max` is zero before and after, *ticket too
+cudaError_t launch_adjoint_absmax(const void* a, size_t n, int adj64, AdjScale* scale, unsigned long long* max,
+                                  unsigned* ticket, cudaStream_t st);
 // dL/d(sigma_D, sigma_N) from the adjoints of lam_D, 1/sigma_D and lam_N
 cudaError_t launch_sigma_grads(const double* dparam, double sigma_D, double sigma_N, double* out, cudaStream_t st);
 
