@@ -307,6 +307,7 @@ dim3 sweep_block() { return dim3(pv::SWEEP_BX, pv::SWEEP_BY); }
 // the sweep kernel of a launch over n_tiles tiles, and its work items
 template <typename T>
 pv::SweepMode sweep_mode(int n_tiles) {
+    if (sizeof(T) == 4 && n_tiles <= pv::ROWS_FEW_TILES) return pv::SWEEP_ROWS_FEW;
     if (n_tiles <= pv::row_mode_tiles<T>()) return pv::SWEEP_ROWS;
     return n_tiles > pv::stream_mode_tiles<T>() ? pv::SWEEP_STREAM : pv::SWEEP_TILES;
 }
@@ -315,6 +316,7 @@ using SweepKernel = decltype(&pv::k_sweeps<T, pv::SWEEP_TILES>);
 template <typename T>
 SweepKernel<T> sweep_kernel(int n_tiles) {
     switch (sweep_mode<T>(n_tiles)) {
+        case pv::SWEEP_ROWS_FEW: return &pv::k_sweeps<T, pv::SWEEP_ROWS_FEW>;
         case pv::SWEEP_ROWS: return &pv::k_sweeps<T, pv::SWEEP_ROWS>;
         case pv::SWEEP_STREAM: return &pv::k_sweeps<T, pv::SWEEP_STREAM>;
         default: return &pv::k_sweeps<T, pv::SWEEP_TILES>;
@@ -322,7 +324,8 @@ SweepKernel<T> sweep_kernel(int n_tiles) {
 }
 template <typename T>
 int sweep_items(int n_tiles) {
-    return sweep_mode<T>(n_tiles) == pv::SWEEP_ROWS ? n_tiles * pv::TILE_H : n_tiles;
+    const pv::SweepMode m = sweep_mode<T>(n_tiles);
+    return m == pv::SWEEP_ROWS || m == pv::SWEEP_ROWS_FEW ? n_tiles * pv::TILE_H : n_tiles;
 }
 
 // dynamic shared memory of the sweep kernels (above the 48 KB default for double)
@@ -331,7 +334,7 @@ cudaError_t sweep_attributes() {
     static cudaError_t once = [] {
         cudaError_t e = cudaSuccess;
         for (SweepKernel<T> k : {&pv::k_sweeps<T, pv::SWEEP_TILES>, &pv::k_sweeps<T, pv::SWEEP_STREAM>,
-                                 &pv::k_sweeps<T, pv::SWEEP_ROWS>})
+                                 &pv::k_sweeps<T, pv::SWEEP_ROWS>, &pv::k_sweeps<T, pv::SWEEP_ROWS_FEW>})
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)pv::sweep_smem_bytes<T>());
@@ -1397,6 +1400,7 @@ pixvod_status batch_sweeps(pixvod_batch* b, int n_iters, int schedule) {
         pv::GridSync gs{sy, sy + 1, sy + 2, b->wait_limit};
         int grid = b->blocks_per_sm * b->num_sms;
         if (grid > sweep_items<T>(b->n_work)) grid = sweep_items<T>(b->n_work);
+        if (sweep_mode<T>(b->n_work) == pv::SWEEP_ROWS_FEW && grid > 3 * b->num_sms) grid = 3 * b->num_sms;  // resident
         const pv::SeqDesc<T>* d = descs<T>(b);
         const pv::Work* w = works(b);
         int n_work = b->n_work, cur0 = cur;
@@ -1603,14 +1607,15 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
     if (s == PIXVOD_OK) {
         int m = 0;
         s = cuda_status(p->precision == 64
-                            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, sweep_kernel<double>(B.n_work),
+                            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, pv::k_sweeps<double, pv::SWEEP_ROWS>,
                                                                             pv::SWEEP_THREADS,
                                                                             pv::sweep_smem_bytes<double>())
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, sweep_kernel<float>(B.n_work),
+                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, pv::k_sweeps<float, pv::SWEEP_ROWS>,
                                                                             pv::SWEEP_THREADS,
                                                                             pv::sweep_smem_bytes<float>()));
         // the persistent schedule runs grid sequences (a quadtree sweep is two
-        // dependent launches)
+        // dependent launches); the rows' kernel stands for all but SWEEP_ROWS_FEW,
+        // whose grid is bounded at the launch
         b->max_blocks_per_sm = coop && !b->qt ? (m < 4 ? m : 4) : 0;
         b->blocks_per_sm = b->max_blocks_per_sm;
         if (b->max_blocks_per_sm < 1) b->schedule = PIXVOD_SCHED_BATCHED;

@@ -46,7 +46,16 @@ constexpr int stream_mode_tiles() {
     return sizeof(T) == 4 ? 608 : 304;
 }
 
-enum SweepMode { SWEEP_TILES, SWEEP_STREAM, SWEEP_ROWS };
+// FP32 rows whose blocks all fit on the SMs at 3 a piece get the registers of three
+// blocks instead of four (64x48 5.9 -> 5.6 us a sweep, 128x96 8.2 -> 6.9; where they no
+// longer fit, 160x120 went 8.6 -> 11.7)
+constexpr int ROWS_FEW_TILES = 152 * 3 / TILE_H;
+
+enum SweepMode { SWEEP_TILES, SWEEP_STREAM, SWEEP_ROWS, SWEEP_ROWS_FEW };
+template <typename T, SweepMode MODE>
+constexpr int sweep_min_blocks() {
+    return sizeof(T) == 8 ? 2 : (MODE == SWEEP_ROWS_FEW ? 3 : 4);
+}
 
 struct Work {
     int seq;
@@ -126,14 +135,14 @@ __device__ __forceinline__ bool grid_sync(const GridSync& gs) {
 // own: with both paths in one, 256x256 took 19.3 us a sweep instead of 18.9 and
 // 2048x1536 837 instead of 821.
 template <typename T, SweepMode MODE>
-__global__ void __launch_bounds__(SWEEP_THREADS, sizeof(T) == 4 ? 4 : 2) k_sweeps(const SeqDesc<T>* __restrict__ seqs,
+__global__ void __launch_bounds__(SWEEP_THREADS, sweep_min_blocks<T, MODE>()) k_sweeps(const SeqDesc<T>* __restrict__ seqs,
                                                              const Work* __restrict__ work, int n_tiles,
                                                              int n_iters, int cur0, int flip0,
                                                              GridSync gs) {
     // msg[p * TILE_PX + tid]: a tile's 84 message Lambda planes, bulk-copied in at the
     // start of the tile (the old messages), overwritten in place by the damped new
     // ones; by rows, the four directions' messages of the row
-    constexpr bool ROWS = MODE == SWEEP_ROWS;
+    constexpr bool ROWS = MODE == SWEEP_ROWS || MODE == SWEEP_ROWS_FEW;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
     if (!ROWS) {

@@ -672,10 +672,10 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
 // its direction's messages and its share of the rest. A tile's latency is one
 // direction's instead of four in turn, on four times as many SMs; that every warp
 // solves the belief costs nothing while the schedulers are idle. Per sweep, by
-// tiles and by rows: 64x48 10.8 and 5.7 us, 128x96 11.4 and 7.7, 160x120 12.6 and
-// 8.2, 224x160 15.0 and 14.1, 256x192 17.2 and 19.6; FP64, bound by its pipe: 64x48
-// 123 and 49, 128x96 123 and 155. Every thread of the block must call it; the caller synchronises
-// the block before `msg` is reused.
+// tiles and by rows: 64x48 10.5 and 5.5 us, 128x96 10.9 and 6.9, 160x120 12.6 and
+// 8.5, 224x160 15.0 and 14.8, 256x192 17.3 and 19.6; FP64, bound by its pipe: 64x48
+// 122 and 49, 128x96 123 and 168. Every thread of the block must call it; the caller
+// synchronises the block before `msg` is reused.
 constexpr int ROW_VALUES = 29;  // a direction's Lambda, eta and normal message in shared memory
 template <typename T>
 __device__ __forceinline__ void sweep_row(const SweepArgs<T>& a, int tx, int ty, int row, T* msg, bool last_sweep) {

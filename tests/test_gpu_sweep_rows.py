@@ -19,8 +19,8 @@ from test_gpu_parity import one_sweep_check, sample_pixels  # noqa: E402
 DEV = torch.device("cuda:0")
 
 
-# tiles of 32 x 4: up to 304 (FP32) or 76 (FP64) are swept by rows
-@pytest.mark.parametrize("prec,size,tiles", [(32, (31, 3), 1), (32, (608, 63), 304), (32, (609, 61), 320),
+# tiles of 32 x 4: up to 304 (FP32; up to 114 with more registers) or 76 (FP64) are swept by rows
+@pytest.mark.parametrize("prec,size,tiles", [(32, (31, 3), 1), (32, (608, 23), 114), (32, (609, 23), 120), (32, (608, 63), 304), (32, (609, 61), 320),
                                              (64, (33, 5), 4), (64, (127, 74), 76), (64, (129, 61), 80)])
 def test_one_sweep_on_both_sides_of_the_rule(prec, size, tiles):
     w, h = size
