@@ -572,9 +572,10 @@ pixvod_status run_sweeps_recorded(pixvod_handle* h, int n) {
 
 template <typename T>
 pixvod_status run_reduce(pixvod_handle* h, int anchor) {
-    launch_pdl(pv::k_reduce<T>, dim3(h->L.tiles_x * h->L.tiles_y), dim3(pv::RED_THREADS), 0, h->stream,
-               geometry<T>(h), state_ptr<T>(h, h->cur), reinterpret_cast<double*>(h->ws + h->L.off_partials),
-               scalars(h), anchor);
+    const int n_tiles = h->L.tiles_x * h->L.tiles_y, per = pv::reduce_group(n_tiles);
+    launch_pdl(pv::k_reduce<T>, dim3((n_tiles + per - 1) / per), dim3(pv::RED_THREADS), 0, h->stream, geometry<T>(h),
+               state_ptr<T>(h, h->cur), reinterpret_cast<double*>(h->ws + h->L.off_partials), scalars(h), anchor,
+               n_tiles);
     return launched(h);
 }
 

@@ -211,7 +211,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_batch_reduce(const SeqDesc<T>* 
                                                               int anchor) {
     const Work wk = work[blockIdx.x];
     const SeqDesc<T>& d = seqs[wk.seq];
-    reduce_tile(d.g, d.state[cur], d.partials, d.sc, anchor, wk.tile, d.n_tiles);
+    const int per = reduce_group(d.n_tiles);
+    if (wk.tile % per == 0) reduce_tiles(d.g, d.state[cur], d.partials, d.sc, anchor, wk.tile / per, d.n_tiles);
 }
 
 }  // namespace pv

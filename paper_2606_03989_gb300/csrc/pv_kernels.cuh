@@ -867,62 +867,98 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs<T>& a, int tx, int ty
 // ---------------------------------------------------------------------------
 constexpr int RED_THREADS = TILE_PX;
 
+// FP64 runs at 1/64 of the FP32 rate here, and the reduction's additions bound it
+// (640x480: 35 of them per thread in a butterfly of all seven sums took 50 us cold).
+// So a block adds up several tiles per thread first, a float is widened by its bits,
+// and the butterfly halves the number of sums a lane holds at each step.
+__device__ __forceinline__ double widen(float x) {
+    const int b = __float_as_int(x), e = (b >> 23) & 0xff;
+    if (e == 0 || e == 0xff) return double(x);
+    return __hiloint2double((b & 0x80000000) | ((e + 896) << 20) | ((b & 0x7fffff) >> 3), b << 29);
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // Seven sums over the block's threads, in a fixed order (shuffles within a warp,
-// then the warps in order), in every thread of warp 0; one barrier where a
-// shared-memory tree took seven.
-__device__ __forceinline__ void block_sum7(double* r, double (*sh)[RED_THREADS / 32]) {
-    __syncthreads();  // sh may still be read from an earlier sum
+// then the warps in order): thread q of the block gets sum q (q < 7, others 0).
+__device__ __forceinline__ double block_sum7(const double* r, double (*sh)[RED_THREADS / 32]) {
+    const int lane = threadIdx.x & 31;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+    double v[4], w[2];
 #pragma unroll
-    for (int q = 0; q < 7; ++q)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) r[q] += __shfl_xor_sync(0xffffffffu, r[q], o);
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-        for (int q = 0; q < 7; ++q) sh[q][threadIdx.x >> 5] = r[q];
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 7; ++q) {
-        r[q] = sh[q][0];
-#pragma unroll
-        for (int w = 1; w < RED_THREADS / 32; ++w) r[q] += sh[q][w];
+    for (int q = 0; q < 4; ++q) {
+        const double lo = r[q], hi = q < 3 ? r[q + 4] : 0.0;
+        v[q] = (b4 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b4 ? lo : hi, 16);
     }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        w[q] = (b3 ? v[q + 2] : v[q]) + __shfl_xor_sync(0xffffffffu, b3 ? v[q] : v[q + 2], 8);
+    double x = (b2 ? w[1] : w[0]) + __shfl_xor_sync(0xffffffffu, b2 ? w[0] : w[1], 4);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    const int q = lane >> 2;  // the sum this lane holds
+    __syncthreads();          // sh may still be read from an earlier sum
+    if ((lane & 3) == 0 && q < 7) sh[q][threadIdx.x >> 5] = x;
+    __syncthreads();
+    double y = 0.0;
+    if (threadIdx.x < 7) {
+        y = sh[threadIdx.x][0];
+#pragma unroll
+        for (int k = 1; k < RED_THREADS / 32; ++k) y += sh[threadIdx.x][k];
+    }
+    return y;
 }
 
-// One block per state tile sums that tile's 7 mean planes (double accumulation,
-// fixed order); the last block to finish sums the tile partials in tile order,
+// Tiles that one block of the reduction adds up: as many as make at most one wave
+// of blocks at 4 per SM.
+__host__ __device__ constexpr int reduce_group(int n_tiles) { return (n_tiles + 607) / 608; }
+
+// The block of group `group` sums its tiles' 7 mean planes (double accumulation,
+// fixed order); the last block to finish sums the groups' partials in order,
 // writes xi_est and the mean log-depth, composes T_cur = Exp(xi_est) T_kf and,
 // at an anchoring frame, moves the keyframe: T_kf <- T_cur, d_prior <- d_mean.
 template <typename T>
-__device__ __forceinline__ void reduce_tile(const Geometry<T>& g, const T* __restrict__ state,
-                                            double* __restrict__ partials, Scalars* sc, int anchor, int tile,
-                                            int n_tiles) {
+__device__ __forceinline__ void reduce_tiles(const Geometry<T>& g, const T* __restrict__ state,
+                                             double* __restrict__ partials, Scalars* sc, int anchor, int group,
+                                             int n_tiles) {
     __shared__ double sh[7][RED_THREADS / 32];
     __shared__ bool last;
     const int tid = threadIdx.x;
-    const int u = (tile % g.tiles_x) * TILE_W + tid % TILE_W;
-    const int v = (tile / g.tiles_x) * TILE_H + tid / TILE_W;
+    const int per = reduce_group(n_tiles), n_groups = (n_tiles + per - 1) / per;
+    const int end = min((group + 1) * per, n_tiles);
     double r[7] = {0, 0, 0, 0, 0, 0, 0};
-    if (u < g.W && v < g.H) {
-        const T* st = state + (size_t)tile * TILE_WORDS + tid;
+#pragma unroll 4
+    for (int tile = group * per; tile < end; ++tile) {
+        const int u = (tile % g.tiles_x) * TILE_W + tid % TILE_W;
+        const int v = (tile / g.tiles_x) * TILE_H + tid / TILE_W;
+        if (u < g.W && v < g.H) {
+            const T* st = state + (size_t)tile * TILE_WORDS + tid;
 #pragma unroll
-        for (int q = 0; q < 7; ++q) r[q] = double(st[q * TILE_PX]);
+            for (int q = 0; q < 7; ++q) r[q] += widen(st[q * TILE_PX]);
+        }
     }
-    block_sum7(r, sh);
-    if (tid == 0) {
-#pragma unroll
-        for (int q = 0; q < 7; ++q) partials[tile * 7 + q] = r[q];
+    double y = block_sum7(r, sh);
+    if (tid < 7) {
+        partials[group * 7 + tid] = y;
         __threadfence();
-        last = atomicAdd(&sc->counter, 1u) == (unsigned)(n_tiles - 1);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(&sc->counter, 1u) == (unsigned)(n_groups - 1);
     }
     __syncthreads();
     if (!last) return;
+    __threadfence();
 #pragma unroll
     for (int q = 0; q < 7; ++q) r[q] = 0.0;
-#pragma unroll 4
-    for (int h = tid; h < n_tiles; h += RED_THREADS)
+#pragma unroll 5
+    for (int h = tid; h < n_groups; h += RED_THREADS)
 #pragma unroll
         for (int q = 0; q < 7; ++q) r[q] += __ldcg(partials + h * 7 + q);
-    block_sum7(r, sh);
+    y = block_sum7(r, sh);
+    if (tid < 32)
+#pragma unroll
+        for (int q = 0; q < 7; ++q) r[q] = __shfl_sync(0xffffffffu, y, q);
     if (tid == 0) {
         const double n = double(g.W) * double(g.H);
         double xi[6], R[9], t[3];
@@ -952,9 +988,9 @@ __device__ __forceinline__ void reduce_tile(const Geometry<T>& g, const T* __res
 template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce(Geometry<T> g, const T* __restrict__ state,
                                                         double* __restrict__ partials, Scalars* sc,
-                                                        int anchor) {
+                                                        int anchor, int n_tiles) {
     pdl_wait();
-    reduce_tile(g, state, partials, sc, anchor, blockIdx.x, gridDim.x);
+    reduce_tiles(g, state, partials, sc, anchor, blockIdx.x, n_tiles);
 }
 
 // Depth output: exp(sign * mu_6) as dense float32.
