@@ -41,6 +41,9 @@ STATE_PLANES, INPUT_PLANES = 151, 6
 # algorithmic bytes per pixel per sweep (FP32): every state plane read once and
 # written once, plus the six input planes (I_s, I_t, g_x, g_y, m_x, m_y) read once
 BYTES_PER_PX_SWEEP = 4 * (2 * STATE_PLANES + INPUT_PLANES)
+# quadtree: three of a pixel's four identity-message slots (27 planes each) hold
+# zeros and are neither read nor written by a sweep
+BYTES_PER_PX_QT = 4 * (2 * (STATE_PLANES - 81) + INPUT_PLANES)
 FALLBACK_HBM_GBS = 6800.0
 PROFILED_SWEEPS = 200   # sweeps timed one by one, after the timed region
 
@@ -552,7 +555,7 @@ def run_quadtree(args):
     node_bytes = 4 * 2 * 162 * n_nodes            # node planes read and written per sweep
     q = out[pv.TOPOLOGY_QUADTREE]
     peak, peak_kind = hbm_peak()
-    bytes_sweep = px * BYTES_PER_PX_SWEEP + node_bytes
+    bytes_sweep = px * BYTES_PER_PX_QT + node_bytes
     achieved = bytes_sweep / (q["sweep_ms"] * 1e-3) / 1e9
     line = {
         "metric": "Mpixel*GBP-sweeps/s at 640x480, quadtree identity topology", "unit": "Mpx*sweeps/s",
