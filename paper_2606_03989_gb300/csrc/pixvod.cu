@@ -710,6 +710,7 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
     A.tape.cap = kTapeCap;
     A.tape.n_slots = R.slots;
     A.adj_max = adj_max;
+    A.ticket = ticket;
     const size_t adj_elems = (size_t)n_tiles * pv::TILE_WORDS;
     const size_t adj_used = adj_elems * (adj64 ? sizeof(double) : sizeof(float));  // of the FP64-sized buffers
     // the prior mean of the segment the frame was tracked in

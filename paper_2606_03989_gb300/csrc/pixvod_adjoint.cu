@@ -63,6 +63,7 @@ struct HwArgs {
     const AdjScale* scale;
     AdjScale* scale_next;
     unsigned long long* adj_max;
+    unsigned* ticket;
 };
 
 template <typename T>
@@ -106,6 +107,7 @@ HwArgs<T> hw_args(const AdjArgs& A) {
     h.scale = A.scale;
     h.scale_next = A.scale_next;
     h.adj_max = A.adj_max;
+    h.ticket = A.ticket;
     return h;
 }
 
@@ -118,6 +120,13 @@ __device__ __forceinline__ double scaled_double(float v, int E, double scale) {
     return __hiloint2double((b & 0x80000000) | (y << 20) | ((b & 0x7fffff) >> 3), b << 29);
 }
 __device__ __forceinline__ double scaled_double(double v, int, double scale) { return v * scale; }
+
+// m = the larger of m and |x|, if x is finite
+template <typename T>
+__device__ __forceinline__ void absmax_acc(T x, T& m) {
+    const T b = v_abs(x);
+    if (b > m && v_finite(b)) m = b;
+}
 
 // I/O of one pixel's reverse pass in the kernel: reads from the state before
 // the sweep and the adjoint of the state after it; adds the input adjoints to
@@ -137,8 +146,8 @@ struct KernelIO {
     T in_scale;        // adj_out is read times this
     int out_exp;       // the FP64 gradients' factor is 2^out_exp
     double out_scale;
-    mutable T ymax;    // largest |adj_out| read (finite), scaled
     T dIs, lamD, isD, lamN;  // one value each in a pixel's pass
+    T amax;                  // largest |value| added to adj_in (finite)
 
     __device__ size_t nbi(int k) const { return DIR ? sj[0] : sj[k]; }
     __device__ T mu(int q) const { return __ldg(Sin + si + q * TILE_PX); }
@@ -147,11 +156,7 @@ struct KernelIO {
     __device__ T nb(int k, int q) const { return __ldg(Sin + nbi(k) + nb_plane(q, k) * TILE_PX); }
     __device__ T I_s() const { return Is; }
     __device__ T tap(int q) const { return tapv[q]; }
-    __device__ T ybar(int q) const {
-        const T y = __ldcg(Ao + si + q * TILE_PX) * in_scale, b = v_abs(y);
-        if (b > ymax && v_finite(b)) ymax = b;
-        return y;
-    }
+    __device__ T ybar(int q) const { return __ldcg(Ao + si + q * TILE_PX) * in_scale; }
     // the stages' scratch (scr_in, scr_out: the pixel's planes)
     const T* scr_in;
     T* scr_out;
@@ -172,10 +177,14 @@ struct KernelIO {
         scr_out[(SCR_CHK + chk_plane(q)) * TILE_PX] = y;
         if (q >= 144 && (q & 1) == 0) scr_out[(SCR_CHK_S + (q - 144) / 2) * TILE_PX] = scale;
     }
-    __device__ void add_mu(int q, T v) { atomicAdd(Ai + si + q * TILE_PX, v); }
-    __device__ void add_msg(int k, int q, T v) { atomicAdd(Ai + si + (PL_ID + ID_STRIDE * k + q) * TILE_PX, v); }
-    __device__ void add_nm(int q, T v) { atomicAdd(Ai + si + (PL_NM + q) * TILE_PX, v); }
-    __device__ void add_nb(int k, int q, T v) { atomicAdd(Ai + nbi(k) + nb_plane(q, k) * TILE_PX, v); }
+    __device__ void add(T* p, T v) {
+        atomicAdd(p, v);
+        absmax_acc(v, amax);
+    }
+    __device__ void add_mu(int q, T v) { add(Ai + si + q * TILE_PX, v); }
+    __device__ void add_msg(int k, int q, T v) { add(Ai + si + (PL_ID + ID_STRIDE * k + q) * TILE_PX, v); }
+    __device__ void add_nm(int q, T v) { add(Ai + si + (PL_NM + q) * TILE_PX, v); }
+    __device__ void add_nb(int k, int q, T v) { add(Ai + nbi(k) + nb_plane(q, k) * TILE_PX, v); }
     __device__ void add_Is(T v) { dIs = v; }
     // taps 0-3 of I_t directly; 4-7 of g_x and 8-11 of g_y through the central
     // differences of the target ingest (replicated borders)
@@ -227,8 +236,7 @@ __device__ bool pixel_context(const HwArgs<T>& A, int tile, int lane, int k, hw:
     io.si = (size_t)tile * TILE_WORDS + lane;
     io.scr_in = nullptr;
     io.scr_out = nullptr;
-    io.dIs = io.lamD = io.isD = io.lamN = T(0);
-    io.ymax = T(0);
+    io.dIs = io.lamD = io.isD = io.lamN = io.amax = T(0);
     // The adjoint state is rescaled by a power of two before every pass: the
     // unrolled derivative can grow by many orders of magnitude over the sweeps,
     // beyond the float range, while the pass is linear in its input.
@@ -428,7 +436,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? PV_ADJ_MAIN_BLOCKS :
     const int tile = blockIdx.x, lane = threadIdx.x;
     __shared__ double red[3][TILE_PX / 32];
     double sums[3] = {0.0, 0.0, 0.0};
-    T ymax = T(0);
+    T amax = T(0);
     KernelIO<T, false> io;
     hw::PixCtx<T> c;
     int u, v;
@@ -486,7 +494,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? PV_ADJ_MAIN_BLOCKS :
         sums[0] = scaled_double(io.lamD, io.out_exp, io.out_scale);
         sums[1] = scaled_double(io.isD, io.out_exp, io.out_scale);
         sums[2] = scaled_double(io.lamN, io.out_exp, io.out_scale);
-        ymax = io.ymax;
+        amax = io.amax;
     }
     // the block's sums (as 384 FP64 atomics on shared memory they were a
     // compare-and-swap loop per lane)
@@ -503,7 +511,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? PV_ADJ_MAIN_BLOCKS :
         for (int w = 0; w < TILE_PX / 32; ++w) x += red[lane][w];
         if (x != 0.0) atomicAdd(A.dparam + lane, x);
     }
-    check_block_max(ymax, A.adj_max);
+    check_block_max(amax, A.adj_max);
     pdl_trigger();
 }
 
@@ -521,7 +529,7 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? 4 : 1) k_adjoint_dir
     hw::PixCtx<T> c;
     int u, v;
     bool has = false;
-    T mm = T(0), ymax = T(0);
+    T mm = T(0), amax = T(0);
     if (pixel_context(A, tile, lane, k, c, io, &u, &v, &has) && has) {
         T* sp = scr + (size_t)tile * SCR_WORDS + lane;
         io.scr_in = sp;
@@ -560,10 +568,10 @@ __global__ void __launch_bounds__(TILE_PX, sizeof(T) == 4 ? 4 : 1) k_adjoint_dir
         hw::identity_vjp(io, c, k, R, t, f, Lb, eb, Rb, tb);
         for (int q = 0; q < 9; ++q) atomicAdd(sp + (SCR_MAIN + hw::MO_RB + q) * TILE_PX, Rb[q]);
         for (int q = 0; q < 3; ++q) atomicAdd(sp + (SCR_MAIN + hw::MO_TB + q) * TILE_PX, tb[q]);
-        ymax = io.ymax;
+        amax = io.amax;
     }
     check_block_max(mm, A.mismatch);
-    check_block_max<1>(ymax, A.adj_max);
+    check_block_max<1>(amax, A.adj_max);
     pdl_trigger();
 }
 
@@ -579,19 +587,17 @@ __device__ __forceinline__ void set_scale(AdjScale* s, double E, double max) {
 }
 
 // Pose stage (last): the pixel's xi adjoint from the (R, t) adjoints of its Exp,
-// the recompute check of what the main stage left (SCR_CHK), and the next pass's
-// factors.
+// the recompute check of what the main stage left (SCR_CHK), and, by the last block,
+// the next pass's factors.
 template <typename T>
 __global__ void __launch_bounds__(TILE_PX) k_adjoint_pose(const HwArgs<T> A, const T* __restrict__ scr) {
     pdl_wait();
     const int tile = blockIdx.x, lane = threadIdx.x;
-    if (tile == 0 && lane == 0)
-        set_scale(A.scale_next, __ldcg(&A.scale->E), __longlong_as_double((long long)atomicExch(A.adj_max, 0ull)));
     KernelIO<T, true> io;
     hw::PixCtx<T> c;
     int u, v;
     bool has = false;
-    T mm = T(0);
+    T mm = T(0), amax = T(0);
     if (pixel_context(A, tile, lane, 0, c, io, &u, &v, &has)) {
         io.scr_in = scr + (size_t)tile * SCR_WORDS + lane;
         T xi[6], Rb[9], tb[3], xib[6];
@@ -622,25 +628,34 @@ __global__ void __launch_bounds__(TILE_PX) k_adjoint_pose(const HwArgs<T> A, con
             scalar(PL_NM + 2 * k, nl, unit_scale(nl));
             scalar(PL_NM + 2 * k + 1, chk(PL_NM + 2 * k + 1), __ldcg(io.scr_in + (SCR_CHK_S + k) * TILE_PX));
         }
+        amax = io.amax;
     }
     check_block_max(mm, A.mismatch);
+    check_block_max<1>(amax, A.adj_max);
+    if (lane == 0) {
+        __threadfence();
+        if (atomicAdd(A.ticket, 1u) == gridDim.x - 1) {
+            __threadfence();
+            set_scale(A.scale_next, __ldcg(&A.scale->E), __longlong_as_double((long long)atomicExch(A.adj_max, 0ull)));
+            *A.ticket = 0u;
+        }
+    }
     pdl_trigger();
 }
 
-// max |a[i]| over finite values, in the adjoint's own precision, with 16-byte
-// loads (n a multiple of 4: the adjoint state is a whole number of 128-pixel
-// tiles)
 __device__ __forceinline__ void absmax_acc(float4 x, float& m) {
-    const float v[4] = {fabsf(x.x), fabsf(x.y), fabsf(x.z), fabsf(x.w)};
-    for (int q = 0; q < 4; ++q)
-        if (isfinite(v[q]) && v[q] > m) m = v[q];
+    absmax_acc(x.x, m);
+    absmax_acc(x.y, m);
+    absmax_acc(x.z, m);
+    absmax_acc(x.w, m);
 }
 __device__ __forceinline__ void absmax_acc(double2 x, double& m) {
-    const double v[2] = {fabs(x.x), fabs(x.y)};
-    for (int q = 0; q < 2; ++q)
-        if (isfinite(v[q]) && v[q] > m) m = v[q];
+    absmax_acc(x.x, m);
+    absmax_acc(x.y, m);
 }
-// Its last block sets the first pass's factors.
+// max |a[i]| of the seed over finite values, in the adjoint's own precision, with
+// 16-byte loads (n a multiple of 4: the adjoint state is a whole number of 128-pixel
+// tiles); the last block sets the first pass's factors.
 template <typename T, typename V>
 __global__ void k_adjoint_absmax(const V* __restrict__ a, size_t nv, AdjScale* __restrict__ scale,
                                  unsigned long long* __restrict__ mx, unsigned* __restrict__ ticket) {

@@ -23,18 +23,17 @@ struct TapeCtl {
 
 constexpr unsigned FLAG_TAPE_FULL = 0x8u;  // a pixel's tape overflowed: its gradient is missing
 
-// Arguments of the adjoint of one sweep. State buffers and input planes hold
-// FP64 when state64 is set, FP32 otherwise. The adjoint states are FP64 for the
-// tape kernel and in the state's precision for the hand-written one; the
-// gradients of the inputs and factor weights are FP64.
 // Rescaling of the adjoint state by a power of two: a pass reads adj_out, in units
 // of 2^(E - e), times 2^-e, so that its adj_in and its gradients are in units of 2^E.
-// For the first pass e = ilogb(max |adj_out|) (launch_adjoint_absmax); each pass
-// leaves the next one's factors, e = ilogb of the largest value it read itself,
-// scaled. That is one pass behind: a pass reads values up to twice the growth of the
-// adjoint over one sweep (6x on the benchmark's frames), far inside the float range,
-// and no pass of its own over the 151 planes is needed (19.5 us of 173 per reverse
-// sweep at 320x240 in FP32).
+// For the first pass e = ilogb(max |adj_out|) (launch_adjoint_absmax); each pass leaves
+// the next one's factors, e = ilogb of the largest single value that it added to
+// adj_in. An entry of adj_in is a sum of at most five of them, so a pass reads values
+// below 2^4 and has the rest of the float range for one sweep's growth; where the five
+// cancel, by at most the 24 bits that their sum has, it reads smaller ones. (The
+// largest value that a pass reads itself is one sweep behind: the state that it writes
+// then holds two sweeps' growth, which overflowed from 2^58 a sweep on. The sums
+// themselves, read back by the last stage, cost 12 us of 155 a reverse sweep at
+// 320x240, these factors 2.)
 struct AdjScale {
     double E;
     double in;      // 2^-e
@@ -43,6 +42,10 @@ struct AdjScale {
     int E32;        // E
 };
 
+// Arguments of the adjoint of one sweep. State buffers and input planes hold
+// FP64 when state64 is set, FP32 otherwise. The adjoint states are FP64 for the
+// tape kernel and in the state's precision for the hand-written one; the
+// gradients of the inputs and factor weights are FP64.
 struct AdjArgs {
     Geometry<double> g;
     int state64;
@@ -65,11 +68,13 @@ struct AdjArgs {
     unsigned* max_nodes;           // longest tape of a pixel
     unsigned* flags;
     ad::TapeCtl tape;
-    // hand-written pass: the factors of this pass and of the one after it, and the
-    // largest |adj_out| this pass reads (as bits)
+    // hand-written pass: the factors of this pass and of the one after it, the largest
+    // value added to adj_in so far (as bits) and the blocks of the last stage that have
+    // put theirs in; both zero before and after a pass
     AdjScale* scale;
     AdjScale* scale_next;
     unsigned long long* adj_max;
+    unsigned* ticket;
 };
 
 // adjoint of one sweep by the reverse-mode tape (FP64), `blocks` blocks of
