@@ -277,7 +277,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity
 
 // Loads of the swept state bypass L1 (ld.global.cg): the persistent batched
 // kernel reads, after a grid barrier, data other SMs wrote in the same launch,
-// and an SM's L1 is not kept coherent with those writes.
+// and an SM's L1 is not kept coherent with those writes. Only for memory that the
+// calling thread has not itself written with plain stores: __ldcg is inline assembly
+// without a memory clobber, so nothing orders it behind them.
 template <typename T>
 __device__ __forceinline__ T ld_state(const T* p) {
     return __ldcg(p);
@@ -622,12 +624,13 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
     T tau[7], qv;
     belief_update(Mp, md, eb, J, alpha, rph, tau, qv, br, flags);
     if (a.br) a.br[tile * TILE_PX + tid] = br;
-    // the new eta, back for the projection below
+    // the new eta, back for the projection below: plain loads, which the compiler keeps
+    // behind the loop's stores (__ldcg does not say that it reads memory)
     T en[24];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int q = 0; q < 6; ++q) en[6 * k + q] = __ldcg(Di + (PL_ID + ID_STRIDE * k + LAM + q) * TILE_PX);
+        for (int q = 0; q < 6; ++q) en[6 * k + q] = Di[(PL_ID + ID_STRIDE * k + LAM + q) * TILE_PX];
     // mu <- mu (+) tau
     {
         T xn[6];
