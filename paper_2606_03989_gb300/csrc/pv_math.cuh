@@ -370,8 +370,8 @@ template <typename T>
 PV_HD void se3_log_q(const T* q, const T* t, T* xi) {
     const T s2 = dot3(q + 1, q + 1);
     T ratio, D;  // theta = ratio v
-    if (s2 < T(QUAT_S2_MAX) && q[0] > T(0)) {
-        ratio = T(2) * asin_series<T, QuatPrec<T>::asin_terms>(s2);
+    if (s2 < T(QUAT_S2_MAX)) {  // of either sign: -q is the same rotation, and v may vanish
+        ratio = (q[0] < T(0) ? T(-2) : T(2)) * asin_series<T, QuatPrec<T>::asin_terms>(s2);
         D = d_series<T, QuatPrec<T>::d_terms>(s2 * (ratio * ratio));
     } else {
         const T s = v_sqrt(s2), w = v_abs(q[0]);
