@@ -221,7 +221,8 @@ struct pixvod_handle {
     int rec_n;           // sweeps of the recorded frame (0: none)
     int rec_window;      // differentiate only the last rec_window sweeps (0: all)
     bool rec_valid;      // the recorded frame can be differentiated
-    bool qt_stale;       // quadtree: the loaded state has values in identity slots 1..3
+    int qt_clear;        // quadtree: sweeps that k_qt_clear still follows, after a load (-1: a batch's
+                         // sequence, which cannot be loaded)
     // profiling
     bool profiling;
     std::vector<cudaEvent_t> ev;
@@ -479,13 +480,22 @@ pixvod_status launch_qt_sweep(pixvod_handle* h) {
     pixvod_status s = launched(h);
     if (s != PIXVOD_OK) return s;
     launch_pdl(pv::k_qt_node_belief<T>, dim3(qt_belief_blocks(h)), dim3(128), 0, h->stream, A, off + 2, 1);
-    if ((s = launched(h)) != PIXVOD_OK || !h->qt_stale) return s;
-    // a loaded checkpoint's unused identity slots, now consumed: zero from here on
-    h->qt_stale = false;
-    return cuda_status(cudaMemset2DAsync(state_ptr<T>(h, h->cur) + (pv::PL_ID + pv::ID_STRIDE) * pv::TILE_PX,
-                                         pv::TILE_WORDS * sizeof(T), 0,
-                                         (pv::MSG_PLANES - pv::ID_STRIDE) * pv::TILE_PX * sizeof(T),
-                                         (size_t)h->L.tiles_x * h->L.tiles_y, h->stream));
+    return launched(h);
+}
+
+// k_qt_clear after the sweep that wrote state buffer `buf`
+template <typename T>
+pixvod_status launch_qt_clear(pixvod_handle* h, int buf) {
+    const int n_tiles = h->L.tiles_x * h->L.tiles_y;
+    launch_pdl(pv::k_qt_clear<T>, dim3(n_tiles < 608 ? n_tiles : 608), dim3(pv::TILE_PX), 0, h->stream, geometry<T>(h),
+               state_ptr<T>(h, buf), scalars(h));
+    return launched(h);
+}
+
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) (void)cudaGetLastError();
+    return c == cudaStreamCaptureStatusActive;
 }
 
 template <typename T>
@@ -493,6 +503,7 @@ pixvod_status run_sweeps(pixvod_handle* h, int n) {
     pixvod_status st = cuda_status(sweep_attributes<T>());
     if (st != PIXVOD_OK) return st;
     const int n_tiles = h->L.tiles_x * h->L.tiles_y;
+    const bool captured = is_quadtree(h) && h->qt_clear >= 0 && capturing(h->stream);  // may be replayed after a load
     for (int it = 0; it < n; ++it) {
         bool prof = h->profiling;
         if (prof) {
@@ -502,6 +513,10 @@ pixvod_status run_sweeps(pixvod_handle* h, int n) {
         pixvod_status s;
         if (is_quadtree(h)) {
             s = launch_qt_sweep<T>(h);
+            if (s == PIXVOD_OK && (captured ? it < 2 : h->qt_clear > 0)) {
+                s = launch_qt_clear<T>(h, h->cur ^ 1);
+                if (!captured) h->qt_clear--;
+            }
         } else {
             launch_sweep<T>(desc_ptr<T>(h), nullptr, n_tiles, h->cur, h->cur, h->stream);
             s = launched(h);
@@ -911,7 +926,7 @@ pixvod_status pixvod_create(const pixvod_intrinsics* K, const pixvod_params* p, 
     h->rec_n = 0;
     h->rec_window = 0;
     h->rec_valid = false;
-    h->qt_stale = false;
+    h->qt_clear = 0;
     pixvod_status s = cuda_status(cudaMemsetAsync(h->ws, 0, L.total, h->stream));
     if (s == PIXVOD_OK) {
         // T_kf = T_cur = identity
@@ -1114,16 +1129,18 @@ pixvod_status pixvod_load_state(pixvod_handle* h, const void* h_buf, size_t byte
         size_t row = (size_t)h->L.q.n_nodes * h->L.elt;
         s = cuda_status(cudaMemcpy2DAsync(h->ws + h->L.off_node[h->cur], h->L.q.stride * h->L.elt, buf + hd[14], row,
                                           row, pv::NODE_PLANES, cudaMemcpyHostToDevice, h->stream));
+        // identity slots 1..3 of this buffer may hold values now, those of the other one
+        // still from an earlier load: the next two sweeps write both
+        const unsigned sweeps = 2;
+        h->qt_clear = 2;
+        if (s == PIXVOD_OK)
+            s = cuda_status(cudaMemcpyAsync(&scalars(h)->qt_clear, &sweeps, sizeof(sweeps), cudaMemcpyHostToDevice,
+                                            h->stream));
         if (s != PIXVOD_OK) return s;
     }
     if ((s = cuda_status(cudaStreamSynchronize(h->stream))) != PIXVOD_OK) return s;
     h->frame_index = hd[7];
     h->has_target = hd[11] == 1;
-    if (is_quadtree(h)) {  // identity slots 1..3 are zero in every state but a foreign one
-        const size_t lo = kHeaderBytes + pb * (pv::PL_ID + pv::ID_STRIDE), hi = kHeaderBytes + pb * pv::PL_NM;
-        h->qt_stale = false;
-        for (size_t k = lo; k < hi && !h->qt_stale; ++k) h->qt_stale = buf[k] != 0;
-    }
     return PIXVOD_OK;
 }
 
@@ -1598,7 +1615,7 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
         h.rec_n = 0;
         h.rec_window = 0;
         h.rec_valid = false;
-        h.qt_stale = false;
+        h.qt_clear = -1;
     }
     int dev = 0;
     s = cuda_status(cudaGetDevice(&dev));

@@ -73,7 +73,9 @@ struct Scalars {
     double d_mean;     // mean log-depth after the last reduction
     unsigned flags;
     unsigned counter;  // last-block ticket of the reduction
-    double pad[6];
+    unsigned qt_clear;   // quadtree: sweeps whose buffer k_qt_clear still has to clear, after a load
+    unsigned qt_ticket;  // blocks of k_qt_clear that have read it
+    double pad[5];
 };
 
 template <typename T>

@@ -2,7 +2,8 @@
 // graph; Sec. 4.2: sigma_R and sigma_P halved per level). Pixels keep the state
 // layout of the grid sweep, using identity slot 0 for the factor to their level-1
 // node (slots 1..3 are zero in both state buffers from the start and are not
-// written: 324 of a pixel's 604 bytes); pose nodes of every level live in one
+// written: 324 of a pixel's 604 bytes; k_qt_clear zeroes what a loaded checkpoint
+// held there); pose nodes of every level live in one
 // structure-of-arrays buffer. One synchronous sweep = k_qt_messages +
 // k_qt_node_belief: the first (pixel updates and the messages into the nodes)
 // reads only the `in` buffers, the second the node messages the first wrote, and
@@ -471,6 +472,35 @@ __global__ void __launch_bounds__(128) k_qt_node_belief(const QtArgs<T>* __restr
     pdl_wait();
     qt_node_belief(A[i], blockIdx.x - __ldg(off + i));
     pdl_trigger();
+}
+
+// After a load, whose blob may hold values in identity slots 1..3: zeros in those of
+// the buffer that the sweep before this kernel has written, while Scalars::qt_clear
+// says that one may hold values. The count is in device memory, so that sweeps
+// captured in a graph before the load clear too when they are replayed. (Tested in
+// the sweep's own kernels it cost every sweep 1 to 2 %: k_qt_messages is at its
+// register limit.) Block = 128 threads; the last one to have read the count lowers it.
+template <typename T>
+__global__ void k_qt_clear(Geometry<T> g, T* __restrict__ state, Scalars* sc) {
+    pdl_wait();
+    const unsigned c = *static_cast<volatile unsigned*>(&sc->qt_clear);
+    if (c) {
+        const int n_tiles = g.tiles_x * ((g.H + TILE_H - 1) / TILE_H), lane = threadIdx.x;
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            const int u = (tile % g.tiles_x) * TILE_W + lane % TILE_W, v = (tile / g.tiles_x) * TILE_H + lane / TILE_W;
+            if (u >= g.W || v >= g.H) continue;
+            T* d = state + (size_t)tile * TILE_WORDS + (PL_ID + ID_STRIDE) * TILE_PX + lane;
+            for (int q = 0; q < MSG_PLANES - ID_STRIDE; ++q) d[q * TILE_PX] = T(0);
+        }
+    }
+    __syncthreads();  // every thread of the block has read the count
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&sc->qt_ticket, 1u) == gridDim.x - 1) {
+            sc->qt_ticket = 0u;
+            if (c) sc->qt_clear = c - 1;
+        }
+    }
 }
 
 // Keyframe reset of every node: identity pose, belief = the level's pose prior,
