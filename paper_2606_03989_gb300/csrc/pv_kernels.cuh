@@ -608,7 +608,7 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
         for (int k = 0; k < 6; ++k)
             if (q == pidx(k, k)) x = F.lam_P;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) x += msg[(LAM * k + q) * TILE_PX + tid];
+        for (int k = 0; k < 4; ++k) x += msg[PV_IDX((LAM * k + q) * TILE_PX + tid, LAM_PLANES * TILE_PX, flags)];
         Mp[q] = x;
     }
     T nl[4], ne[4];
@@ -658,7 +658,7 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const T* mb = msg + (k * LAM) * TILE_PX + tid;
+        const T* mb = msg + PV_IDX((k * LAM) * TILE_PX + tid, (LAM_PLANES - LAM + 1) * TILE_PX, flags);
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
             T e = en[6 * k + r];
@@ -682,6 +682,8 @@ __device__ __forceinline__ bool sweep_pixel(const SweepArgs<T>& a, int tx, int t
 // 122 and 49, 128x96 123 and 168. Every thread of the block must call it; the caller
 // synchronises the block before `msg` is reused.
 constexpr int ROW_VALUES = 29;  // a direction's Lambda, eta and normal message in shared memory
+constexpr int ROW_SLOTS = 4 * ROW_VALUES * TILE_W;
+static_assert(ROW_SLOTS <= LAM_PLANES * TILE_PX, "the rows' values fit the sweep's shared memory");
 template <typename T>
 __device__ __forceinline__ void sweep_row(const SweepArgs<T>& a, int tx, int ty, int row, T* msg, bool last_sweep) {
     const int k = threadIdx.y, x = threadIdx.x;
@@ -698,7 +700,7 @@ __device__ __forceinline__ void sweep_row(const SweepArgs<T>& a, int tx, int ty,
     const int i = inside ? (int)PV_IDX(v * g.pitch + u, g.plane, flags) : 0;
     const T* __restrict__ Si = a.in + PV_IDX(tile * TILE_WORDS + lane, n_state, flags);
     T* __restrict__ Di = a.out + PV_IDX(tile * TILE_WORDS + lane, n_state, flags);
-    T* sh = msg + k * ROW_VALUES * TILE_W + x;  // this direction's values
+    T* sh = msg + PV_IDX(k * ROW_VALUES * TILE_W + x, ROW_SLOTS - (ROW_VALUES - 1) * TILE_W, flags);  // this direction's values
     T xi[6], d = T(0), qi[4], t[3];
     T alpha = T(0), rph = T(0), J[7];
     unsigned char br = 0;
@@ -751,7 +753,7 @@ __device__ __forceinline__ void sweep_row(const SweepArgs<T>& a, int tx, int ty,
         for (int j = 0; j < 6; ++j)
             if (q == pidx(j, j)) y = F.lam_P;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) y += msg[(j * ROW_VALUES + q) * TILE_W + x];
+        for (int j = 0; j < 4; ++j) y += msg[PV_IDX((j * ROW_VALUES + q) * TILE_W + x, ROW_SLOTS, flags)];
         Mp[q] = y;
     }
 #pragma unroll
@@ -759,7 +761,7 @@ __device__ __forceinline__ void sweep_row(const SweepArgs<T>& a, int tx, int ty,
     eb[6] = -mul_rn(F.lam_Z, d - T(a.sc->d_prior));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const T* sj = msg + j * ROW_VALUES * TILE_W + x;
+        const T* sj = msg + PV_IDX(j * ROW_VALUES * TILE_W + x, ROW_SLOTS - (ROW_VALUES - 1) * TILE_W, flags);
 #pragma unroll
         for (int q = 0; q < 6; ++q) eb[q] += sj[(LAM + q) * TILE_W];
         md += sj[27 * TILE_W];
