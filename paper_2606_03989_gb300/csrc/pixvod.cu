@@ -209,6 +209,7 @@ struct pixvod_handle {
     Layout L;
     char* ws;
     cudaStream_t stream;
+    int num_sms;
     int cur;  // state buffer holding the current state
     int64_t frame_index;
     bool has_target;
@@ -305,27 +306,19 @@ dim3 pixel_grid(const pixvod_handle* h) {
 }
 dim3 sweep_block() { return dim3(pv::SWEEP_BX, pv::SWEEP_BY); }
 
-// the sweep kernel of a launch over n_tiles tiles, and its work items
-template <typename T>
-pv::SweepMode sweep_mode(int n_tiles) {
-    if (sizeof(T) == 4 && n_tiles <= pv::ROWS_FEW_TILES) return pv::SWEEP_ROWS_FEW;
-    if (n_tiles <= pv::row_mode_tiles<T>()) return pv::SWEEP_ROWS;
-    return n_tiles > pv::stream_mode_tiles<T>() ? pv::SWEEP_STREAM : pv::SWEEP_TILES;
-}
+// the kernel of a sweep mode (ROWS_FEW and STREAM are FP32 modes), and the blocks of
+// a launch over n_tiles tiles
 template <typename T>
 using SweepKernel = decltype(&pv::k_sweeps<T, pv::SWEEP_TILES>);
 template <typename T>
-SweepKernel<T> sweep_kernel(int n_tiles) {
-    switch (sweep_mode<T>(n_tiles)) {
-        case pv::SWEEP_ROWS_FEW: return &pv::k_sweeps<T, pv::SWEEP_ROWS_FEW>;
-        case pv::SWEEP_ROWS: return &pv::k_sweeps<T, pv::SWEEP_ROWS>;
-        case pv::SWEEP_STREAM: return &pv::k_sweeps<T, pv::SWEEP_STREAM>;
-        default: return &pv::k_sweeps<T, pv::SWEEP_TILES>;
+SweepKernel<T> sweep_kernel(pv::SweepMode m) {
+    if constexpr (sizeof(T) == 4) {
+        if (m == pv::SWEEP_ROWS_FEW) return &pv::k_sweeps<T, pv::SWEEP_ROWS_FEW>;
+        if (m == pv::SWEEP_STREAM) return &pv::k_sweeps<T, pv::SWEEP_STREAM>;
     }
+    return m == pv::SWEEP_ROWS ? &pv::k_sweeps<T, pv::SWEEP_ROWS> : &pv::k_sweeps<T, pv::SWEEP_TILES>;
 }
-template <typename T>
-int sweep_items(int n_tiles) {
-    const pv::SweepMode m = sweep_mode<T>(n_tiles);
+int sweep_items(pv::SweepMode m, int n_tiles) {
     return m == pv::SWEEP_ROWS || m == pv::SWEEP_ROWS_FEW ? n_tiles * pv::TILE_H : n_tiles;
 }
 
@@ -334,22 +327,30 @@ template <typename T>
 cudaError_t sweep_attributes() {
     static cudaError_t once = [] {
         cudaError_t e = cudaSuccess;
-        for (SweepKernel<T> k : {&pv::k_sweeps<T, pv::SWEEP_TILES>, &pv::k_sweeps<T, pv::SWEEP_STREAM>,
-                                 &pv::k_sweeps<T, pv::SWEEP_ROWS>, &pv::k_sweeps<T, pv::SWEEP_ROWS_FEW>})
+        for (pv::SweepMode m : {pv::SWEEP_TILES, pv::SWEEP_STREAM, pv::SWEEP_ROWS, pv::SWEEP_ROWS_FEW})
             if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                e = cudaFuncSetAttribute(sweep_kernel<T>(m), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)pv::sweep_smem_bytes<T>());
         return e;
     }();
     return once;
 }
 
+// blocks per SM of a mode's kernel (its shared memory set by sweep_attributes)
+template <typename T>
+cudaError_t sweep_occupancy(pv::SweepMode m, int* blocks) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, sweep_kernel<T>(m), pv::SWEEP_THREADS,
+                                                         pv::sweep_smem_bytes<T>());
+}
+
 // one synchronous grid sweep: the tiles of `work` (null: of the descriptor's
 // sequence in order; from the end when `flip` is odd), reading state buffer `cur`
 template <typename T>
-void launch_sweep(const pv::SeqDesc<T>* desc, const pv::Work* work, int n_tiles, int cur, int flip, cudaStream_t st) {
-    launch_pdl(sweep_kernel<T>(n_tiles), dim3(sweep_items<T>(n_tiles)), sweep_block(), pv::sweep_smem_bytes<T>(), st,
-               desc, work, n_tiles, 1, cur, flip, pv::GridSync{nullptr, nullptr, nullptr, 0});
+void launch_sweep(const pv::SeqDesc<T>* desc, const pv::Work* work, int n_tiles, int num_sms, int cur, int flip,
+                  cudaStream_t st) {
+    const pv::SweepMode m = pv::sweep_mode<T>(n_tiles, num_sms);
+    launch_pdl(sweep_kernel<T>(m), dim3(sweep_items(m, n_tiles)), sweep_block(), pv::sweep_smem_bytes<T>(), st, desc,
+               work, n_tiles, 1, cur, flip, pv::GridSync{nullptr, nullptr, nullptr, 0});
 }
 
 pixvod_status cuda_status(cudaError_t e) {
@@ -518,7 +519,7 @@ pixvod_status run_sweeps(pixvod_handle* h, int n) {
                 if (!captured) h->qt_clear--;
             }
         } else {
-            launch_sweep<T>(desc_ptr<T>(h), nullptr, n_tiles, h->cur, h->cur, h->stream);
+            launch_sweep<T>(desc_ptr<T>(h), nullptr, n_tiles, h->num_sms, h->cur, h->cur, h->stream);
             s = launched(h);
         }
         if (prof) {
@@ -569,7 +570,7 @@ pixvod_status run_sweeps_recorded(pixvod_handle* h, int n) {
         if (s != PIXVOD_OK) return s;
         const pv::SeqDesc<T>* dd = reinterpret_cast<const pv::SeqDesc<T>*>(h->rec_ws + R.off_desc);
         for (int c = 1; c <= n; ++c) {
-            launch_sweep<T>(dd + (c - 1), nullptr, n_tiles, 0, c, h->stream);
+            launch_sweep<T>(dd + (c - 1), nullptr, n_tiles, h->num_sms, 0, c, h->stream);
             if ((s = launched(h)) != PIXVOD_OK) return s;
         }
         h->cur = cur0 ^ 1;
@@ -777,7 +778,7 @@ pixvod_status backward_impl(pixvod_handle* h, const double* g_xi, const double* 
         const int c = seg * k, len = n - c < k ? n - c : k;
         if (c + len <= first) break;
         for (int j = 1; j <= len; ++j) {
-            launch_sweep<T>(ddesc + (c + j - 1), nullptr, n_tiles, 0, j, st);
+            launch_sweep<T>(ddesc + (c + j - 1), nullptr, n_tiles, h->num_sms, 0, j, st);
             if ((s = launched(h)) != PIXVOD_OK) return s;
         }
         for (int j = len; j >= 1 && c + j > first; --j)
@@ -927,7 +928,11 @@ pixvod_status pixvod_create(const pixvod_intrinsics* K, const pixvod_params* p, 
     h->rec_window = 0;
     h->rec_valid = false;
     h->qt_clear = 0;
-    pixvod_status s = cuda_status(cudaMemsetAsync(h->ws, 0, L.total, h->stream));
+    h->num_sms = 0;
+    int dev = 0;
+    pixvod_status s = cuda_status(cudaGetDevice(&dev));
+    if (s == PIXVOD_OK) s = cuda_status(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev));
+    if (s == PIXVOD_OK) s = cuda_status(cudaMemsetAsync(h->ws, 0, L.total, h->stream));
     if (s == PIXVOD_OK) {
         // T_kf = T_cur = identity
         double eye[16] = {1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1};
@@ -1272,7 +1277,8 @@ struct pixvod_batch {
     int n_work;
     int schedule;
     int blocks_per_sm;
-    int max_blocks_per_sm;
+    int max_blocks_per_sm;  // that a caller may ask for
+    int resident_blocks;    // that a launch of the batch's own sweep kernel may hold
     int num_sms;
     long long wait_limit;   // polls of the grid barrier before it gives up
     bool barrier_fault;     // test hook: arrival counter starts at 1 (pixvod_batch_inject_barrier_fault)
@@ -1403,7 +1409,7 @@ pixvod_status batch_sweeps(pixvod_batch* b, int n_iters, int schedule) {
         }
     } else if (schedule == PIXVOD_SCHED_BATCHED) {
         for (int it = 0; it < n_iters; ++it) {
-            launch_sweep<T>(descs<T>(b), works(b), b->n_work, cur, cur, b->stream);
+            launch_sweep<T>(descs<T>(b), works(b), b->n_work, b->num_sms, cur, cur, b->stream);
             if ((s = batch_launched(b)) != PIXVOD_OK) return s;
             cur ^= 1;
         }
@@ -1417,14 +1423,15 @@ pixvod_status batch_sweeps(pixvod_batch* b, int n_iters, int schedule) {
             (s = cuda_status(cudaMemsetAsync(reinterpret_cast<char*>(sy) + 3, 1, 1, b->stream))) != PIXVOD_OK)
             return s;
         pv::GridSync gs{sy, sy + 1, sy + 2, b->wait_limit};
+        const pv::SweepMode mode = pv::sweep_mode<T>(b->n_work, b->num_sms);
         int grid = b->blocks_per_sm * b->num_sms;
-        if (grid > sweep_items<T>(b->n_work)) grid = sweep_items<T>(b->n_work);
-        if (sweep_mode<T>(b->n_work) == pv::SWEEP_ROWS_FEW && grid > 3 * b->num_sms) grid = 3 * b->num_sms;  // resident
+        if (grid > b->resident_blocks) grid = b->resident_blocks;
+        if (grid > sweep_items(mode, b->n_work)) grid = sweep_items(mode, b->n_work);
         const pv::SeqDesc<T>* d = descs<T>(b);
         const pv::Work* w = works(b);
         int n_work = b->n_work, cur0 = cur;
         void* args[] = {(void*)&d, (void*)&w, (void*)&n_work, (void*)&n_iters, (void*)&cur0, (void*)&cur0, (void*)&gs};
-        s = cuda_status(cudaLaunchCooperativeKernel((const void*)sweep_kernel<T>(n_work), dim3(grid), sweep_block(),
+        s = cuda_status(cudaLaunchCooperativeKernel((const void*)sweep_kernel<T>(mode), dim3(grid), sweep_block(),
                                                     args, pv::sweep_smem_bytes<T>(), b->stream));
         b->launches++;
         if (s != PIXVOD_OK) return s;
@@ -1624,18 +1631,19 @@ pixvod_status pixvod_batch_create(int32_t n, const pixvod_intrinsics* K, const p
     if (s == PIXVOD_OK) s = cuda_status(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
     if (s == PIXVOD_OK) s = cuda_status(p->precision == 64 ? sweep_attributes<double>() : sweep_attributes<float>());
     if (s == PIXVOD_OK) {
-        int m = 0;
-        s = cuda_status(p->precision == 64
-                            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, pv::k_sweeps<double, pv::SWEEP_ROWS>,
-                                                                            pv::SWEEP_THREADS,
-                                                                            pv::sweep_smem_bytes<double>())
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, pv::k_sweeps<float, pv::SWEEP_ROWS>,
-                                                                            pv::SWEEP_THREADS,
-                                                                            pv::sweep_smem_bytes<float>()));
+        for (auto& h : b->seq) h.num_sms = b->num_sms;
         // the persistent schedule runs grid sequences (a quadtree sweep is two
-        // dependent launches); the rows' kernel stands for all but SWEEP_ROWS_FEW,
-        // whose grid is bounded at the launch
-        b->max_blocks_per_sm = coop && !b->qt ? (m < 4 ? m : 4) : 0;
+        // dependent launches). A caller may ask for as many blocks per SM as the rows'
+        // kernel has; a launch holds no more than are resident of its own kernel.
+        int m = 0, own = 0;
+        s = cuda_status(p->precision == 64 ? sweep_occupancy<double>(pv::SWEEP_ROWS, &m)
+                                           : sweep_occupancy<float>(pv::SWEEP_ROWS, &m));
+        if (s == PIXVOD_OK)
+            s = cuda_status(p->precision == 64
+                                ? sweep_occupancy<double>(pv::sweep_mode<double>(b->n_work, b->num_sms), &own)
+                                : sweep_occupancy<float>(pv::sweep_mode<float>(b->n_work, b->num_sms), &own));
+        b->resident_blocks = own * b->num_sms;
+        b->max_blocks_per_sm = coop && !b->qt && own > 0 ? (m < 4 ? m : 4) : 0;
         b->blocks_per_sm = b->max_blocks_per_sm;
         if (b->max_blocks_per_sm < 1) b->schedule = PIXVOD_SCHED_BATCHED;
     }

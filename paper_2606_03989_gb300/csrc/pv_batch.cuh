@@ -26,32 +26,28 @@ struct SeqDesc {
     int n_tiles;
 };
 
-// A launch over at most this many tiles (of one image, or of a batch together) sweeps
-// them by rows (sweep_row): two tiles per SM in FP32 (measured: faster at 280 tiles,
-// slower at 384), half a tile in FP64 (the rows then fit on the SMs at once; faster at
-// 24 and 48 tiles, slower at 96).
-template <typename T>
-constexpr int row_mode_tiles() {
-    return sizeof(T) == 4 ? 304 : 76;
-}
-
-// A launch over more tiles than this marks the new state's plane stores to leave L2
-// first: one wave of tiles in FP32 (4 blocks on 152 SMs), whose two buffers (94 MB)
-// L2 still holds in the next sweep. Larger states do not stay anyway, and what is
-// evicted is then rather the output than the neighbours' planes still to be read: a
-// sweep at 320x240 20.5 and 21.1 us without and with, 333x251 30.9 and 30.5, 512x384
-// 58.7 and 57.4, 640x480 86.5 and 85.2, 2048x1536 821 and 796; FP64 the same to 0.2 %.
-template <typename T>
-constexpr int stream_mode_tiles() {
-    return sizeof(T) == 4 ? 608 : 304;
-}
-
-// FP32 rows whose blocks all fit on the SMs at 3 a piece get the registers of three
-// blocks instead of four (64x48 5.9 -> 5.6 us a sweep, 128x96 8.2 -> 6.9; where they no
-// longer fit, 160x120 went 8.6 -> 11.7)
-constexpr int ROWS_FEW_TILES = 152 * 3 / TILE_H;
-
+// The sweep kernel of a launch over n_tiles tiles (of one image, or of a batch
+// together) on num_sms SMs. The limits in tiles are those of the 152 SMs measured.
+//  - FP32, up to 3/4 tile per SM (114): rows whose blocks all fit on the SMs at three a
+//    piece get the registers of three (64x48 5.9 -> 5.5 us a sweep, 128x96 8.2 -> 6.9;
+//    where they no longer fit, 160x120 went 8.6 -> 11.7);
+//  - up to 2 tiles per SM (304), in FP64 half a tile (76: the rows then fit on the SMs
+//    at once): rows (sweep_row). FP32 measured faster at 280 tiles, slower at 384; FP64
+//    faster at 24 and 48, slower at 96;
+//  - FP32, above 4 tiles per SM (608): tiles whose plane stores are marked to leave L2
+//    first. Up to there, one wave of 4 blocks per SM, the two buffers (94 MB) are still
+//    in L2 in the next sweep. Larger states do not stay anyway, and what is evicted is
+//    then rather the output than the neighbours' planes still to be read: a sweep at
+//    320x240 20.5 and 21.1 us without and with, 333x251 30.9 and 30.5, 512x384 58.7 and
+//    57.4, 640x480 86.5 and 85.2, 2048x1536 821 and 796 (FP64 the same to 0.2 %).
 enum SweepMode { SWEEP_TILES, SWEEP_STREAM, SWEEP_ROWS, SWEEP_ROWS_FEW };
+template <typename T>
+inline SweepMode sweep_mode(int n_tiles, int num_sms) {
+    if (sizeof(T) == 8) return 2 * n_tiles <= num_sms ? SWEEP_ROWS : SWEEP_TILES;
+    if (n_tiles * TILE_H <= 3 * num_sms) return SWEEP_ROWS_FEW;
+    if (n_tiles <= 2 * num_sms) return SWEEP_ROWS;
+    return n_tiles > 4 * num_sms ? SWEEP_STREAM : SWEEP_TILES;
+}
 template <typename T, SweepMode MODE>
 constexpr int sweep_min_blocks() {
     return sizeof(T) == 8 ? 2 : (MODE == SWEEP_ROWS_FEW ? 3 : 4);

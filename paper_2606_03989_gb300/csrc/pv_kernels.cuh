@@ -916,7 +916,8 @@ __device__ __forceinline__ double block_sum7(const double* r, double (*sh)[RED_T
 }
 
 // Tiles that one block of the reduction adds up: as many as make at most one wave
-// of blocks at 4 per SM.
+// of blocks at 4 on each of 152 SMs. A constant on every device: it sets the order of
+// the sums.
 __host__ __device__ constexpr int reduce_group(int n_tiles) { return (n_tiles + 607) / 608; }
 
 // The block of group `group` sums its tiles' 7 mean planes (double accumulation,
