@@ -492,12 +492,11 @@ PV_HD void photometric(T d, T I_s, const T* tap, const PixCtx<T>& c, const T* R,
 
 // What the reverse pass of an identity message needs from its forward: the
 // residual rb, W = M_p,j - Lambda_j->i, C^-1 (packed; C = W + lam_R I + u u^T)
-// and eta_new (ID_FWD_VALS values, in this order).
+// and eta_new.
 template <typename T>
 struct IdFwd {
     T rb[6], W[21], Ci[21], en[6];
 };
-constexpr int ID_FWD_VALS = 54;
 
 // The damped identity message of direction k into the pixel at pose (q, t) =
 // Exp(io.mu): Lambda (packed) and eta, from the neighbour's values and the pixel's
