@@ -300,7 +300,7 @@ __device__ __forceinline__ void st_state(T* p, T x) {
 // Thread block of the sweep kernel: one state tile (32 x 4 pixels), one thread
 // per pixel; 4 blocks per SM (43 KB of shared memory and at most 128 registers
 // each). What a tile waits on is memory latency (at 640x480 about 34 of the 46
-// thousand clocks that it took; no pipe or bandwidth above 45 %), so loads are
+// thousand clocks that it took; DRAM at 47 % and no pipe above 30), so loads are
 // issued early and together and the register file holds as many pixels as it can:
 //  - the four messages' Lambda are bulk-copied into shared memory, damped in place
 //    and bulk-copied out; M_p is summed from there after the loop instead of in 21
